@@ -63,8 +63,8 @@ typedef enum qtea_option {
   QTEA_OPT_RESIDUAL_FP8 = 2, /* residual_vals holds FP8 E4M3 bytes [N/4][s] (Sec. 4.1), passed
                                 through the same pointer argument */
   QTEA_OPT_FIXED_POINT = 4,  /* base-3 layouts: batch-1 calls decode by the fixed-point
-                                dot-product kernel instead of the paper's sign-symmetric lookup
-                                table (Sec. 3.5, Appendix A), the default */
+                                dot-product kernel instead of the default (the tensor-core kernel, or
+                                the paper's sign-symmetric lookup table, see qtea_pack_layout) */
   QTEA_OPT_STREAM_K = 8      /* 2-bit layouts: batch-1 calls always take the stream-K kernel, never
                                 the row-resident one (see qtea_gemv_grouped) */
 } qtea_option;
@@ -101,11 +101,12 @@ typedef enum qtea_option {
  * some problem has K > 4096 or more than 256 salient columns;
  * a latency-bound form for small calls), else the persistent stream-K launch; the tensor-core
  * low-batch kernel takes those at M >= 2 and 2-bit layouts with FP8 residual values (groups of 128
- * columns, or beta absent) at any M; base-3 layouts
- * at M = 1 run on the paper's table-lookup decode (Sec. 3.5, Appendix A); base-3 layouts at
- * 2 <= M <= 4 (or at M = 1 with QTEA_OPT_FIXED_POINT) run on a kernel that stages v*x once per CTA
- * in fixed point (the base-3 problems of a grouped call share one launch); the rest run on general
- * kernels.
+ * columns, or beta absent) at any M; base-3 layouts run on the tensor-core base-3 kernel at any M, but
+ * for the following: at M = 1 with QTEA_OPT_FIXED_POINT on a kernel that stages v*x once per CTA in
+ * fixed point; layouts with so many salient columns that a 512-column chunk's share exceeds 32 of them
+ * on the paper's table-lookup decode (M = 1; Sec. 3.5, Appendix A), that fixed-point kernel (M <= 4) or
+ * a general kernel; the rest run on general kernels. The problems of a grouped call that the same
+ * kernel serves share launches.
  *
  * The call validates every code on the device and synchronizes `stream` once to read the
  * result; invalid codes give QTEA_ERR_BAD_CODES and no layout. It allocates the packed
@@ -148,8 +149,10 @@ int qtea_pack_layout(const int8_t* ternary_codes, int N, int K, int group_size, 
  * (qtea_set_activation_precision); block sums, alpha and the residual are combined in fp32. At 2 <= M <= 16, and for 2-bit layouts in the paper's
  * storage at any M, the tensor cores take 2T*v and x in fp16 (both exact, which needs |v| < 32768)
  * with exact fp32 products and fp32 sums; alpha, beta and the residual are applied in fp32.
- * Base-3 layouts at M <= 4 (when v*x of the call fits in shared memory): the ternary sum is
- * accumulated exactly in integers over 128-column blocks, with v*x in fixed point relative to the
+ * Base-3 layouts on the tensor-core kernel: 2T and v*x (as an fp16 pair whose sum is exact to 22 bits
+ * of the largest of its 512 columns) are exact, products are summed on the tensor cores over at most
+ * 512 columns, the rest in fp32 (infinities and NaN in v*x make the batch row NaN). On the fixed-point
+ * kernel (when v*x of the call fits in shared memory): the ternary sum is accumulated exactly in integers over 128-column blocks, with v*x in fixed point relative to the
  * block's largest |v*x| (|X| < 2^23) after up to 3 massive values per block are taken out and
  * added exactly in fp32; block sums, alpha, beta and the residual are combined in fp32. Other
  * layouts and batch sizes: fp32 throughout.
@@ -192,7 +195,8 @@ typedef enum qtea_kernel {
   QTEA_KERNEL_LOW_BATCH = 4,    /* tensor-core low-batch kernel (2-bit codes) */
   QTEA_KERNEL_BASE3_FIXED = 5,  /* base-3 codes, v*x staged once per CTA in fixed point */
   QTEA_KERNEL_PAPER = 6,        /* general kernel for the paper's storage */
-  QTEA_KERNEL_GENERIC = 7       /* general kernel */
+  QTEA_KERNEL_GENERIC = 7,      /* general kernel */
+  QTEA_KERNEL_BASE3_MMA = 8     /* tensor-core kernel for base-3 codes, any M */
 } qtea_kernel;
 
 /*
@@ -318,9 +322,8 @@ int qtea_set_activation_precision(qtea_layout* layout, int bits);
 /*
  * Storage options of the scales and residual values qtea_gemv reads with this layout: any
  * combination of QTEA_OPT_BIAS and QTEA_OPT_RESIDUAL_FP8 (0 restores fp16 alpha only and fp16
- * residual values), and QTEA_OPT_FIXED_POINT for base-3 layouts (at M = 1 base-3 layouts decode by
- * table lookup unless this option asks for the fixed-point kernel; at 2 <= M <= 4 they always use
- * the fixed-point kernel). Other bits -> QTEA_ERR_INVALID_ARG.
+ * residual values), and QTEA_OPT_FIXED_POINT for base-3 layouts (at M = 1 they decode by the
+ * fixed-point kernel when this option asks for it). Other bits -> QTEA_ERR_INVALID_ARG.
  * With QTEA_OPT_BIAS or QTEA_OPT_RESIDUAL_FP8 set, calls leave the batch-1 kernel (see
  * qtea_pack_layout for which kernel serves which storage); QTEA_OPT_FIXED_POINT changes nothing for
  * 2-bit layouts. Set it before the calls that use it; it takes effect for calls made afterwards.

@@ -271,7 +271,7 @@ def qtea_gemv_grouped(problems, stream=None):
 
 
 QTEA_KERNEL_NAMES = {0: "none", 1: "rows", 2: "stream_k", 3: "lut", 4: "low_batch", 5: "base3_fixed", 6: "paper",
-                     7: "generic"}
+                     7: "generic", 8: "base3_mma"}
 
 
 def qtea_gemv_plan(problems) -> list:

@@ -43,6 +43,7 @@ void release(qtea_layout* l) {
   if (l->mb_gbar) cudaFree(l->mb_gbar);
   if (l->mb_part) cudaFree(l->mb_part);
   if (l->mb_counters) cudaFree(l->mb_counters);
+  if (l->x_part) cudaFree(l->x_part);
   if (l->lut_ws) cudaFree(l->lut_ws);
   if (l->lut_counters) cudaFree(l->lut_counters);
   delete l;
@@ -127,6 +128,33 @@ int plan_m1(qtea_layout* l, const cudaDeviceProp& prop) {
   return QTEA_OK;
 }
 
+// Resources of the tensor-core kernel for a base-3 layout: the partial rows of split tiles. Taken when
+// no chunk's share of the salient entries exceeds what a unit stages.
+int plan_b3mma(qtea_layout* l, const cudaDeviceProp& prop) {
+  l->x_ok = false;
+  if (l->N == 0 || l->K == 0) return QTEA_OK;
+  const int n_chunks = (l->K + kXChunkCols - 1) / kXChunkCols, steps = (l->n_salient + 15) / 16;
+  if ((steps + n_chunks - 1) / n_chunks > kXResSteps || n_chunks > kXMaxChunks || prop.multiProcessorCount > kMaxGrid)
+    return QTEA_OK;
+  if (x_smem_bytes(4, 144, 2) > prop.sharedMemPerBlockOptin || b3mma_configure(prop.sharedMemPerBlockOptin) != cudaSuccess) {
+    cudaGetLastError();
+    return QTEA_OK;
+  }
+  if (l->row_bytes % 16 == 0) {  // else the codes come by 16-byte copies
+    PFN_cuTensorMapEncodeTiled_v12000 encode = get_encode_tiled();
+    cuuint64_t dims[2] = {(cuuint64_t)l->row_bytes, (cuuint64_t)l->N}, strides[1] = {(cuuint64_t)l->row_bytes};
+    cuuint32_t box[2] = {(cuuint32_t)kXBoxBytes, (cuuint32_t)kXTileRows}, estr[2] = {1, 1};
+    l->x_tma = encode && encode(&l->tmap, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, l->packed, dims, strides, box, estr,
+                                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  }
+  const size_t bytes = (size_t)l->sm_count * kXPartWordsPerSm * sizeof(uint32_t);
+  if (cudaMalloc(&l->x_part, bytes) != cudaSuccess) return QTEA_ERR_ALLOC;
+  if (cudaMemset(l->x_part, 0, bytes) != cudaSuccess) return QTEA_ERR_CUDA;
+  l->x_ok = true;
+  return QTEA_OK;
+}
+
 // Resources of the table-lookup kernel for a base-3 layout: split-tile workspace and counters.
 int plan_lut(qtea_layout* l, const cudaDeviceProp& prop) {
   l->lut_ok = false;
@@ -205,6 +233,80 @@ int run_lut(const qtea_gemv_problem* qs, const int* idx, int n, cudaStream_t st)
     if (grid > kMaxGrid) grid = kMaxGrid;
     for (int b = 0; b <= grid; ++b) P.cta_u0[b] = (int)unit_begin_of(b, P.total_units, grid);
     if (launch_lut(P, grouped, grid, st) != cudaSuccess) return QTEA_ERR_CUDA;
+    i += k;
+  }
+  return QTEA_OK;
+}
+
+// The tensor-core base-3 kernel takes this problem: base-3 codes at any batch, unless the fixed-point
+// kernel is asked for at M = 1.
+bool b3mma_eligible(const qtea_layout* l, int M) {
+  return l->x_ok && l->format == QTEA_FMT_BASE3 && !(M == 1 && (l->options & QTEA_OPT_FIXED_POINT));
+}
+
+// Tensor-core base-3 problems: up to kMaxProblems per launch.
+int run_b3mma(const qtea_gemv_problem* qs, const int* idx, int n, int M, cudaStream_t st) {
+  for (int i = 0; i < n;) {
+    const qtea_layout* l0 = qs[idx[i]].packed_ternary;
+    XParams P;
+    std::memset(&P, 0, sizeof(P));
+    P.M = M;
+    P.status = l0->status;
+    P.row_slot = 112;
+    P.tma = 1;
+    TensorMaps maps;
+    std::memset(&maps, 0, sizeof(maps));
+    long long units = 0;
+    int k = 0;
+    for (; i + k < n && k < kMaxProblems; ++k) {
+      const qtea_gemv_problem& q = qs[idx[i + k]];
+      const qtea_layout* l = q.packed_ternary;
+      if (l->sm_count != l0->sm_count) break;  // the partial rows are sized by the SM count
+      XProblem& a = P.prob[k];
+      a.x = q.x;
+      a.packed = l->packed;
+      a.scales = q.row_scale;
+      a.v = q.col_scale;
+      a.sal = q.salient_idx;
+      a.rvals = q.residual_vals;
+      a.ridx = q.residual_idx;
+      a.y = q.y;
+      a.part = l->x_part;
+      a.N = l->N;
+      a.K = l->K;
+      a.s = l->n_salient;
+      a.row_bytes = l->row_bytes;
+      a.n_blocks = l->K_pad / 128;
+      a.n_tiles = (l->N + kXTileRows - 1) / kXTileRows;
+      a.n_chunks = (l->K + kXChunkCols - 1) / kXChunkCols;
+      a.fp8 = (l->options & QTEA_OPT_RESIDUAL_FP8) ? 1 : 0;
+      a.G = l->group_size == l->K ? 1 : a.n_blocks;
+      a.bias = (l->options & QTEA_OPT_BIAS) ? 1 : 0;
+      a.scales_vec = a.bias && a.G % 4 == 0 && aligned(q.row_scale, 16);
+      a.xv_vec = a.K % 8 == 0 && aligned(q.x, 16) && aligned(q.col_scale, 16);
+      a.res_vec = a.s % (a.fp8 ? 8 : 4) == 0 && aligned(q.residual_vals, 8);
+      const long long u = (long long)a.n_tiles * a.n_chunks;
+      if (k > 0 && units + u >= (1ll << 30)) break;
+      if (u >= (1ll << 30)) return QTEA_ERR_UNSUPPORTED;
+      a.res_q = (a.s + 15) / 16 / a.n_chunks;
+      a.res_r = (a.s + 15) / 16 % a.n_chunks;
+      a.unit_begin = (int)units;
+      units += u;
+      if (l->x_tma) std::memcpy(&maps.m[k], &l->tmap, sizeof(CUtensorMap));
+      else P.tma = 0;
+      // a row starts at most 8 bytes past a 16-byte boundary, or anywhere even
+      if (a.row_bytes % 8 != 0) P.row_slot = 144;
+    }
+    P.n_problems = k;
+    P.total_units = (int)units;
+    const int mt = x_mt(M);
+    int S = kXMaxStages;
+    while (S > 2 && x_smem_bytes(mt, P.row_slot, S) > l0->smem_optin) --S;
+    P.n_stages = S;
+    int grid = l0->sm_count;
+    if (units < grid) grid = (int)units;
+    for (int b = 0; b <= grid; ++b) P.cta_u0[b] = (int)unit_begin_of(b, units, grid);
+    if (launch_b3mma(maps, P, grid, x_smem_bytes(mt, P.row_slot, S), st) != cudaSuccess) return QTEA_ERR_CUDA;
     i += k;
   }
   return QTEA_OK;
@@ -892,7 +994,8 @@ int qtea_pack_layout(const int8_t* ternary_codes, int N, int K, int group_size, 
   l->paper_staged_ok = paper_configure(prop.sharedMemPerBlockOptin) == cudaSuccess;
   if (!l->paper_staged_ok) cudaGetLastError();
   l->packed_bytes = (size_t)N * (size_t)l->row_bytes;
-  if (cudaMalloc(&l->packed, l->packed_bytes > 0 ? l->packed_bytes : 16) != cudaSuccess ||
+  // 16 bytes more: the base-3 kernel copies whole 16-byte vectors
+  if (cudaMalloc(&l->packed, l->packed_bytes + 16) != cudaSuccess ||
       cudaMalloc(&l->status, 2 * sizeof(int)) != cudaSuccess) {
     cudaGetLastError();
     release(l);
@@ -915,7 +1018,8 @@ int qtea_pack_layout(const int8_t* ternary_codes, int N, int K, int group_size, 
   } else if (format == QTEA_FMT_2BIT) {
     rc = plan_m1(l, prop);  // the batch-1 and low-batch kernels' resources
   } else {
-    rc = plan_lut(l, prop);  // the table-lookup kernel's resources
+    rc = plan_b3mma(l, prop);  // the tensor-core base-3 kernel's, else the table-lookup kernel's
+    if (rc == QTEA_OK && !l->x_ok) rc = plan_lut(l, prop);
   }
   if (rc == QTEA_OK && cudaStreamSynchronize(st) != cudaSuccess) rc = QTEA_ERR_CUDA;
   if (rc != QTEA_OK) {
@@ -930,13 +1034,14 @@ int qtea_pack_layout(const int8_t* ternary_codes, int N, int K, int group_size, 
 namespace {
 
 // Which path serves problem q at batch M (before the batch-1 choice between the two launch forms).
-enum Route { kRouteNone, kRouteZero, kRouteBatch1, kRouteLut, kRouteMb, kRouteB3, kRoutePaper, kRouteGeneric };
+enum Route { kRouteNone, kRouteZero, kRouteBatch1, kRouteB3Mma, kRouteLut, kRouteMb, kRouteB3, kRoutePaper, kRouteGeneric };
 
 Route route(const qtea_gemv_problem& q, int M) {
   const qtea_layout* l = q.packed_ternary;
   if (l->N == 0) return kRouteNone;
   if (l->K == 0) return kRouteZero;
   if (M == 1 && l->m1_ok && m1_capable(l)) return kRouteBatch1;
+  if (b3mma_eligible(l, M)) return kRouteB3Mma;
   if (lut_eligible(l, M)) return kRouteLut;
   if (mb_capable(l, M)) return kRouteMb;
   if (is_paper(l)) return b3_eligible(paper_params(q, M)) ? kRouteB3 : kRoutePaper;
@@ -965,8 +1070,8 @@ int qtea_gemv_grouped(const qtea_gemv_problem* problems, int n_problems, int M, 
   if (n_problems > 0 && !m1_idx) return QTEA_ERR_ALLOC;
   int* mb_idx = m1_idx + n_problems;
   int b3_idx[8];
-  int n_m1 = 0, n_mb = 0, n_b3 = 0, n_lut = 0;
-  int lut_idx[kMaxProblems];
+  int n_m1 = 0, n_mb = 0, n_b3 = 0, n_lut = 0, n_x = 0;
+  int lut_idx[kMaxProblems], x_idx[kMaxProblems];
   for (int i = 0; i < n_problems && rc == QTEA_OK; ++i) {
     const qtea_gemv_problem& q = problems[i];
     switch (route(q, M)) {
@@ -978,6 +1083,13 @@ int qtea_gemv_grouped(const qtea_gemv_problem* problems, int n_problems, int M, 
         break;
       case kRouteBatch1:
         m1_idx[n_m1++] = i;
+        break;
+      case kRouteB3Mma:
+        x_idx[n_x++] = i;
+        if (n_x == kMaxProblems) {
+          rc = run_b3mma(problems, x_idx, n_x, M, st);
+          n_x = 0;
+        }
         break;
       case kRouteLut:
         lut_idx[n_lut++] = i;
@@ -1005,6 +1117,7 @@ int qtea_gemv_grouped(const qtea_gemv_problem* problems, int n_problems, int M, 
     }
   }
   if (rc == QTEA_OK && n_b3 > 0) rc = run_b3(problems, b3_idx, n_b3, M, st);
+  if (rc == QTEA_OK && n_x > 0) rc = run_b3mma(problems, x_idx, n_x, M, st);
   if (rc == QTEA_OK && n_lut > 0) rc = run_lut(problems, lut_idx, n_lut, st);
   if (rc == QTEA_OK && n_m1 > 0) rc = run_batch1(problems, m1_idx, n_m1, st);
   if (rc == QTEA_OK && n_mb > 0) rc = run_mb(problems, mb_idx, n_mb, M, st);
@@ -1028,6 +1141,7 @@ int qtea_gemv_plan(const qtea_gemv_problem* problems, int n_problems, int M, int
         if (n_m1 < kMaxProblems) m1_idx[n_m1++] = i;
         else m1_many = true;
         break;
+      case kRouteB3Mma: kernels[i] = QTEA_KERNEL_BASE3_MMA; break;
       case kRouteLut: kernels[i] = QTEA_KERNEL_LUT; break;
       case kRouteMb: kernels[i] = QTEA_KERNEL_LOW_BATCH; break;
       case kRouteB3: kernels[i] = QTEA_KERNEL_BASE3_FIXED; break;
