@@ -251,7 +251,7 @@ void qtea_free(qtea_layout* layout);
  *                  group of four rows and salient column, the largest W - W^ and its position
  *
  * Decisions are taken in fp32 with every sum in index order, so the outputs are reproducible bit
- * for bit. Asynchronous on `stream`; scratch (about 16 K + 8 N G bytes) comes from the
+ * for bit. Asynchronous on `stream`; scratch (about 8 K + 16 N G bytes) comes from the
  * stream-ordered allocator.
  * Limits: 1 <= N <= 2^20, 1 <= K <= 65536; W and hdiag 4-byte aligned, row_scale, col_scale and
  * residual_vals 2-byte aligned, salient_idx 4-byte aligned. Returns QTEA_ERR_INVALID_ARG or
