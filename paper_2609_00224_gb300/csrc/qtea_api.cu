@@ -49,6 +49,13 @@ void release(qtea_layout* l) {
   delete l;
 }
 
+// The tensor-core kernel with staged B operands takes a layout of this shape: no chunk's share of the salient
+// entries exceeds what a unit stages.
+bool x_shape_ok(const qtea_layout* l, const cudaDeviceProp& prop) {
+  const int n_chunks = (l->K + kXChunkCols - 1) / kXChunkCols, steps = (l->n_salient + 15) / 16;
+  return (steps + n_chunks - 1) / n_chunks <= kXResSteps && n_chunks <= kXMaxChunks && prop.multiProcessorCount <= kMaxGrid;
+}
+
 // Resources of the batch-1 kernel for one layout: its TMA descriptor (512-row x 512-column
 // units, two 256-row boxes each) and the split-tile workspace.
 int plan_m1(qtea_layout* l, const cudaDeviceProp& prop) {
@@ -99,7 +106,9 @@ int plan_m1(qtea_layout* l, const cudaDeviceProp& prop) {
     l->mb_ok = mb_configure(prop.sharedMemPerBlockOptin, &mb_dyn) == cudaSuccess &&
                mb_prep_configure(prop.sharedMemPerBlockOptin) == cudaSuccess;
     l->prep_smem_optin = prop.sharedMemPerBlockOptin;
-    if (!l->mb_ok) cudaGetLastError();
+    l->mma2_ok = l->mb_ok && x_shape_ok(l, prop) && x_smem_bytes(3, 2, kChunkRowBytes, 2) <= prop.sharedMemPerBlockOptin &&
+                 mma2_configure(prop.sharedMemPerBlockOptin) == cudaSuccess;
+    if (!l->mb_ok || !l->mma2_ok) cudaGetLastError();
     l->mb_smem_optin = mb_dyn;
     if (l->mb_ok) {
       if (cudaMalloc(&l->mb_ws, ws) != cudaSuccess ||
@@ -133,10 +142,8 @@ int plan_m1(qtea_layout* l, const cudaDeviceProp& prop) {
 int plan_b3mma(qtea_layout* l, const cudaDeviceProp& prop) {
   l->x_ok = false;
   if (l->N == 0 || l->K == 0) return QTEA_OK;
-  const int n_chunks = (l->K + kXChunkCols - 1) / kXChunkCols, steps = (l->n_salient + 15) / 16;
-  if ((steps + n_chunks - 1) / n_chunks > kXResSteps || n_chunks > kXMaxChunks || prop.multiProcessorCount > kMaxGrid)
-    return QTEA_OK;
-  if (x_smem_bytes(4, 144, 2) > prop.sharedMemPerBlockOptin || b3mma_configure(prop.sharedMemPerBlockOptin) != cudaSuccess) {
+  if (!x_shape_ok(l, prop)) return QTEA_OK;
+  if (x_smem_bytes(1, 4, 144, 2) > prop.sharedMemPerBlockOptin || b3mma_configure(prop.sharedMemPerBlockOptin) != cudaSuccess) {
     cudaGetLastError();
     return QTEA_OK;
   }
@@ -244,15 +251,23 @@ bool b3mma_eligible(const qtea_layout* l, int M) {
   return l->x_ok && l->format == QTEA_FMT_BASE3 && !(M == 1 && (l->options & QTEA_OPT_FIXED_POINT));
 }
 
-// Tensor-core base-3 problems: up to kMaxProblems per launch.
-int run_b3mma(const qtea_gemv_problem* qs, const int* idx, int n, int M, cudaStream_t st) {
+// 2-bit codes at M >= 2, and at M = 1 what the batch-1 kernels do not take.
+bool mma2_eligible(const qtea_layout* l) { return l->mma2_ok && l->format == QTEA_FMT_2BIT; }
+// Scales staged per unit: groups of 128 columns, or beta.
+bool mma2_grp(const qtea_layout* l) { return l->group_size != l->K || (l->options & QTEA_OPT_BIAS); }
+
+// Problems of the tensor-core kernel with staged B operands, of one format: up to kMaxProblems per launch
+// (2-bit ones with and without staged scales in launches of their own).
+int run_mma(const qtea_gemv_problem* qs, const int* idx, int n, bool base3, int M, cudaStream_t st) {
   for (int i = 0; i < n;) {
     const qtea_layout* l0 = qs[idx[i]].packed_ternary;
+    const bool grp = base3 || mma2_grp(l0);
     XParams P;
     std::memset(&P, 0, sizeof(P));
     P.M = M;
     P.status = l0->status;
-    P.row_slot = 112;
+    for (int k = 0; k < 8; ++k) P.shift[k] = 1u << (14 - 2 * k);
+    P.row_slot = base3 ? 112 : kChunkRowBytes;
     P.tma = 1;
     TensorMaps maps;
     std::memset(&maps, 0, sizeof(maps));
@@ -262,6 +277,7 @@ int run_b3mma(const qtea_gemv_problem* qs, const int* idx, int n, int M, cudaStr
       const qtea_gemv_problem& q = qs[idx[i + k]];
       const qtea_layout* l = q.packed_ternary;
       if (l->sm_count != l0->sm_count) break;  // the partial rows are sized by the SM count
+      if (!base3 && mma2_grp(l) != grp) break;
       XProblem& a = P.prob[k];
       a.x = q.x;
       a.packed = l->packed;
@@ -271,18 +287,18 @@ int run_b3mma(const qtea_gemv_problem* qs, const int* idx, int n, int M, cudaStr
       a.rvals = q.residual_vals;
       a.ridx = q.residual_idx;
       a.y = q.y;
-      a.part = l->x_part;
+      a.part = base3 ? l->x_part : reinterpret_cast<uint32_t*>(l->mb_part);
       a.N = l->N;
       a.K = l->K;
       a.s = l->n_salient;
       a.row_bytes = l->row_bytes;
-      a.n_blocks = l->K_pad / 128;
+      a.n_blocks = (l->K + 127) / 128;
       a.n_tiles = (l->N + kXTileRows - 1) / kXTileRows;
       a.n_chunks = (l->K + kXChunkCols - 1) / kXChunkCols;
       a.fp8 = (l->options & QTEA_OPT_RESIDUAL_FP8) ? 1 : 0;
       a.G = l->group_size == l->K ? 1 : a.n_blocks;
       a.bias = (l->options & QTEA_OPT_BIAS) ? 1 : 0;
-      a.scales_vec = a.bias && a.G % 4 == 0 && aligned(q.row_scale, 16);
+      a.scales_vec = a.G % 4 == 0 && aligned(q.row_scale, a.bias ? 16 : 8);
       a.xv_vec = a.K % 8 == 0 && aligned(q.x, 16) && aligned(q.col_scale, 16);
       a.res_vec = a.s % (a.fp8 ? 8 : 4) == 0 && aligned(q.residual_vals, 8);
       const long long u = (long long)a.n_tiles * a.n_chunks;
@@ -292,21 +308,23 @@ int run_b3mma(const qtea_gemv_problem* qs, const int* idx, int n, int M, cudaStr
       a.res_r = (a.s + 15) / 16 % a.n_chunks;
       a.unit_begin = (int)units;
       units += u;
-      if (l->x_tma) std::memcpy(&maps.m[k], &l->tmap, sizeof(CUtensorMap));
+      if (!base3 || l->x_tma) std::memcpy(&maps.m[k], &l->tmap, sizeof(CUtensorMap));
       else P.tma = 0;
-      // a row starts at most 8 bytes past a 16-byte boundary, or anywhere even
-      if (a.row_bytes % 8 != 0) P.row_slot = 144;
+      // a base-3 row starts at most 8 bytes past a 16-byte boundary, or anywhere even
+      if (base3 && a.row_bytes % 8 != 0) P.row_slot = 144;
     }
     P.n_problems = k;
     P.total_units = (int)units;
-    const int mt = x_mt(M);
+    const int mode = x_mode(base3, M), mt = x_mt(mode, M);
     int S = kXMaxStages;
-    while (S > 2 && x_smem_bytes(mt, P.row_slot, S) > l0->smem_optin) --S;
+    while (S > 2 && x_smem_bytes(mode, mt, P.row_slot, S) > l0->x_smem_optin) --S;
     P.n_stages = S;
     int grid = l0->sm_count;
     if (units < grid) grid = (int)units;
     for (int b = 0; b <= grid; ++b) P.cta_u0[b] = (int)unit_begin_of(b, units, grid);
-    if (launch_b3mma(maps, P, grid, x_smem_bytes(mt, P.row_slot, S), st) != cudaSuccess) return QTEA_ERR_CUDA;
+    const size_t smem = x_smem_bytes(mode, mt, P.row_slot, S);
+    if ((base3 ? launch_b3mma(maps, P, grid, smem, st) : launch_mma2(maps, P, grp, grid, smem, st)) != cudaSuccess)
+      return QTEA_ERR_CUDA;
     i += k;
   }
   return QTEA_OK;
@@ -991,6 +1009,7 @@ int qtea_pack_layout(const int8_t* ternary_codes, int N, int K, int group_size, 
   l->sm_count = prop.multiProcessorCount;
   l->smem_optin = prop.sharedMemPerBlockOptin;
   l->smem_per_sm = prop.sharedMemPerMultiprocessor;
+  l->x_smem_optin = prop.sharedMemPerBlockOptin;
   l->paper_staged_ok = paper_configure(prop.sharedMemPerBlockOptin) == cudaSuccess;
   if (!l->paper_staged_ok) cudaGetLastError();
   l->packed_bytes = (size_t)N * (size_t)l->row_bytes;
@@ -1034,7 +1053,7 @@ int qtea_pack_layout(const int8_t* ternary_codes, int N, int K, int group_size, 
 namespace {
 
 // Which path serves problem q at batch M (before the batch-1 choice between the two launch forms).
-enum Route { kRouteNone, kRouteZero, kRouteBatch1, kRouteB3Mma, kRouteLut, kRouteMb, kRouteB3, kRoutePaper, kRouteGeneric };
+enum Route { kRouteNone, kRouteZero, kRouteBatch1, kRouteB3Mma, kRouteMma2, kRouteLut, kRouteMb, kRouteB3, kRoutePaper, kRouteGeneric };
 
 Route route(const qtea_gemv_problem& q, int M) {
   const qtea_layout* l = q.packed_ternary;
@@ -1043,6 +1062,7 @@ Route route(const qtea_gemv_problem& q, int M) {
   if (M == 1 && l->m1_ok && m1_capable(l)) return kRouteBatch1;
   if (b3mma_eligible(l, M)) return kRouteB3Mma;
   if (lut_eligible(l, M)) return kRouteLut;
+  if (mma2_eligible(l)) return kRouteMma2;
   if (mb_capable(l, M)) return kRouteMb;
   if (is_paper(l)) return b3_eligible(paper_params(q, M)) ? kRouteB3 : kRoutePaper;
   return kRouteGeneric;
@@ -1070,8 +1090,8 @@ int qtea_gemv_grouped(const qtea_gemv_problem* problems, int n_problems, int M, 
   if (n_problems > 0 && !m1_idx) return QTEA_ERR_ALLOC;
   int* mb_idx = m1_idx + n_problems;
   int b3_idx[8];
-  int n_m1 = 0, n_mb = 0, n_b3 = 0, n_lut = 0, n_x = 0;
-  int lut_idx[kMaxProblems], x_idx[kMaxProblems];
+  int n_m1 = 0, n_mb = 0, n_b3 = 0, n_lut = 0, n_x = 0, n_m2 = 0;
+  int lut_idx[kMaxProblems], x_idx[kMaxProblems], m2_idx[kMaxProblems];
   for (int i = 0; i < n_problems && rc == QTEA_OK; ++i) {
     const qtea_gemv_problem& q = problems[i];
     switch (route(q, M)) {
@@ -1087,7 +1107,7 @@ int qtea_gemv_grouped(const qtea_gemv_problem* problems, int n_problems, int M, 
       case kRouteB3Mma:
         x_idx[n_x++] = i;
         if (n_x == kMaxProblems) {
-          rc = run_b3mma(problems, x_idx, n_x, M, st);
+          rc = run_mma(problems, x_idx, n_x, true, M, st);
           n_x = 0;
         }
         break;
@@ -1096,6 +1116,13 @@ int qtea_gemv_grouped(const qtea_gemv_problem* problems, int n_problems, int M, 
         if (n_lut == kMaxProblems) {
           rc = run_lut(problems, lut_idx, n_lut, st);
           n_lut = 0;
+        }
+        break;
+      case kRouteMma2:
+        m2_idx[n_m2++] = i;
+        if (n_m2 == kMaxProblems) {
+          rc = run_mma(problems, m2_idx, n_m2, false, M, st);
+          n_m2 = 0;
         }
         break;
       case kRouteMb:
@@ -1117,7 +1144,8 @@ int qtea_gemv_grouped(const qtea_gemv_problem* problems, int n_problems, int M, 
     }
   }
   if (rc == QTEA_OK && n_b3 > 0) rc = run_b3(problems, b3_idx, n_b3, M, st);
-  if (rc == QTEA_OK && n_x > 0) rc = run_b3mma(problems, x_idx, n_x, M, st);
+  if (rc == QTEA_OK && n_x > 0) rc = run_mma(problems, x_idx, n_x, true, M, st);
+  if (rc == QTEA_OK && n_m2 > 0) rc = run_mma(problems, m2_idx, n_m2, false, M, st);
   if (rc == QTEA_OK && n_lut > 0) rc = run_lut(problems, lut_idx, n_lut, st);
   if (rc == QTEA_OK && n_m1 > 0) rc = run_batch1(problems, m1_idx, n_m1, st);
   if (rc == QTEA_OK && n_mb > 0) rc = run_mb(problems, mb_idx, n_mb, M, st);
@@ -1143,6 +1171,7 @@ int qtea_gemv_plan(const qtea_gemv_problem* problems, int n_problems, int M, int
         break;
       case kRouteB3Mma: kernels[i] = QTEA_KERNEL_BASE3_MMA; break;
       case kRouteLut: kernels[i] = QTEA_KERNEL_LUT; break;
+      case kRouteMma2:
       case kRouteMb: kernels[i] = QTEA_KERNEL_LOW_BATCH; break;
       case kRouteB3: kernels[i] = QTEA_KERNEL_BASE3_FIXED; break;
       case kRoutePaper: kernels[i] = QTEA_KERNEL_PAPER; break;

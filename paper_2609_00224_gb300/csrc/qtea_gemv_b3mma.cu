@@ -1,888 +1,24 @@
-// Tensor-core QTEA GEMV for base-3 layouts (the paper's storage, Sec. 3.5) at 1 <= M <= 16.
-//
-// Computes Eq. 10 (alpha, and optionally beta, per row or per row and 128-column group) plus Eq. 11 on
-// mma.sync m16n8k16 (fp16 operands, fp32 accumulation), with every operand exact:
-//  * Unit of work: 256 rows x 512 columns (four 128-column blocks, 104 code bytes per row). No byte is
-//    decoded twice: at M = 1 lane q of a quad decodes block q of its rows, at M >= 2 the four lanes share
-//    each block's first 24 bytes, six each, and take the last two of one block each.
-//  * A (weights): two code bytes sit in the 16-bit halves of a register, r = 203 * byte < 2^16. The
-//    top two bits of a half are then the byte's highest base-3 digit (203 / 49152 exceeds 1/243 by
-//    less than 1.5e-5, and 242 * 1.5e-5 < 1/243, so no digit is ever off), and three times the other
-//    fourteen bits is the same number for the next digit. ~r & 0xC000C000 turns the two digits
-//    c = T + 1 into the fp16 pair 2T = -2, -0 or +2 (sign bit and top exponent bit).
-//  * B (activations): v*x is exact in fp32; times 2^E (E per chunk and batch row, so that the largest
-//    is below 2^14 after the halving that 2T asks for) it is held as two fp16 columns, hi and lo, whose
-//    sum is exact. Four batch rows make one n8 tile. The sums are folded with 2^-E per chunk.
-//  * Scales: at M = 1 column pair q of the tile is non-zero only in the k slots of lane q, so that a
-//    thread's accumulators hold its own block's sums; at M >= 2 the accumulators are folded per block.
-//    Either way alpha, and beta times the block's sum of x, are applied in fp32 (but for the last two
-//    bytes of a block at M >= 2: there A is alpha * 2T, one exact fp16 multiply).
-//  * Residual (Eq. 11): virtual columns, one per salient column, in steps of 16 spread over the
-//    chunks: A holds the value where the stored position is the row and 0 elsewhere, B holds x.
-// What bounds it: the logic pipe and the MMAs. A weight costs one and a half issued lanes of digit
-// extraction, most of them on the logic pipe (64 lanes per clock per SM); that alone would run at 59
-// weights per clock per SM, the MMAs of one n8 tile alone (new A registers every time: 10.9 cycles each per
-// sub-partition) at 94, both together at 50, whether with 8 or 16 decoding warps. M > 4 adds MMAs.
-// Work split: the units of every problem of a group form one sequence split evenly over one persistent
-// CTA per SM; a tile whose units span several CTAs is finished by the CTA holding its first unit, which
-// reaches it last and adds the others' partial rows in CTA order (self-validating words, as in the
-// other stream-K kernels): results do not depend on timing. 256-row units: 512-row ones left 9 % of the
-// Llama3-8B layer's time to CTAs with one unit more.
-// CTA: eight consumer warps (two 16-row blocks each), and two sets of four helper warps that prepare the
-// units in turn, up to four ahead: the codes (TMA, or 16-byte copies where a row is not a whole number
-// of 16-byte vectors), the scales and the residual (copies), and the B operand, built from x and v in
-// the CTA that uses it, so that neither a pass before the kernel nor a barrier across the grid is needed.
-// The helpers come first in the CTA and their global loads go out a unit ahead: one set of four, or loads
-// where they are used, made the consumers wait 1000 to 4000 cycles per unit.
-// Measured (Llama3-8B layer in the paper's storage, seven GEMVs in one call): M = 1 82.4 -> 32.8 us (table
-// lookup before), M = 4 273 -> 37.1 us (fixed-point dp4a before), M = 16 6440 -> 69 us (the general kernel).
-#include <cuda_fp16.h>
-
-#include "qtea_internal.h"
+// The tensor-core kernel's base-3 forms (see qtea_mma.h): M = 1, and M >= 2 in one to four n8 tiles.
+#include "qtea_mma.h"
 
 namespace qtea {
-namespace {
-
-
-// Partial rows of split tiles are stored XOR-ed with this NaN bit pattern, so that zeroed memory
-// reads as "not written yet" and every word validates itself.
-constexpr uint32_t kXPartEmpty = 0x7FBADBADu;
-
-__device__ __forceinline__ void x_mma(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint2 b) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b.x), "r"(b.y));
-}
-__device__ __forceinline__ void x_mma_first(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint2 b) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
-      : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b.x), "r"(b.y), "f"(0.f));
-}
-__device__ __forceinline__ uint32_t x_hmul2(uint32_t a, uint32_t b) {
-  uint32_t d;
-  asm("mul.rn.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-  return d;
-}
-__device__ __forceinline__ void x_cp16(uint32_t dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-// Eight bytes, the last 8 - n of them zero (n = 8 or 0).
-__device__ __forceinline__ void x_cp8(uint32_t dst, const void* src, int n) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
-}
-// Arrival on `bar` once this thread's earlier cp.async copies have landed (counted in the barrier).
-__device__ __forceinline__ void x_cp_arrive(uint32_t bar) {
-  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ uint32_t x_part_load(const uint32_t* p) {
-  uint32_t w;
-  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(w) : "l"(p) : "memory");
-  return w;
-}
-__device__ __forceinline__ void x_part_store(uint32_t* p, uint32_t w) {
-  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(w) : "memory");
-}
-
-// CTA whose range contains unit u (the inverse of the balanced split cta_u0[b] = b * total / grid).
-__device__ __forceinline__ int x_unit_owner(long long u, long long total, int grid) {
-  return (int)(((u + 1) * grid - 1) / total);
-}
-
-// A unit's problem, tile and chunk. The ceil(s / 16) steps of 16 salient entries are spread over a
-// tile's chunks: chunk ch takes steps [ch nb / n, (ch + 1) nb / n), here rs and its remainder.
-struct XPos {
-  int p, t, ch, rs, rem;
-};
-__device__ __forceinline__ XPos x_pos(const XProblem* tab, int n_problems, int u) {
-  int p = 0;
-  while (p + 1 < n_problems && u >= tab[p + 1].unit_begin) ++p;
-  const int v = u - tab[p].unit_begin, nc = tab[p].n_chunks, t = v / nc, ch = v - t * nc;
-  const int e = ch * (tab[p].res_q * nc + tab[p].res_r), rs = e / nc;  // below 2 kXMaxChunks^2
-  return {p, t, ch, rs, e - rs * nc};
-}
-__device__ __forceinline__ int x_res_steps(const XPos& c, const XProblem& a) {
-  return a.res_q + (c.rem + a.res_r >= a.n_chunks ? 1 : 0);
-}
-__device__ __forceinline__ void x_next(XPos& c, const XProblem* tab) {
-  const XProblem& a = tab[c.p];
-  c.rs += a.res_q;
-  c.rem += a.res_r;
-  if (c.rem >= a.n_chunks) {
-    c.rem -= a.n_chunks;
-    ++c.rs;
-  }
-  if (++c.ch == a.n_chunks) {
-    c.ch = c.rs = c.rem = 0;
-    if (++c.t == a.n_tiles) {
-      c.t = 0;
-      ++c.p;
-    }
-  }
-}
-
-// ---------------------------------------------------------------- helpers
-
-// The unit's code bytes: row r of the tile is copied from the 16-byte boundary at or below its first
-// byte, so that it starts at its own offset (0 .. 14, even) in its slot of row_slot bytes. (Rows of whole
-// 16-byte vectors come by TMA instead, with the same offsets, 0 or 8.)
-template <int H>
-__device__ __forceinline__ void x_issue_codes(const XProblem& a, const XPos& c, uint32_t dst, int row_slot,
-                                              int ht) {
-  const int r0 = ht >> 3, j = ht & 7;
-  const int bytes = 26 * min(4, a.n_blocks - 4 * c.ch);
-  const size_t start = (size_t)(c.t * kXTileRows + r0) * a.row_bytes + (size_t)c.ch * kXChunkBytes;
-  const int off = (int)(start & 15);  // the same for every 8th row: 8 row_bytes is a multiple of 16
-  const uint8_t* src = a.packed + (start - off) + 16 * j;
-  dst += r0 * row_slot + 16 * j;
-  const int rows = a.N - c.t * kXTileRows - r0;
-  constexpr int kRows = H * 4;  // rows per pass
-  const size_t step = (size_t)kRows * a.row_bytes;
-  if (16 * j < off + bytes) {
-#pragma unroll 4
-    for (int r = 0; r < kXTileRows; r += kRows)
-      if (r < rows) x_cp16(dst + r * row_slot, src + (size_t)(r / kRows) * step);
-  }
-}
-
-// Where column c of a block goes in the B operand of a tile: bits 0 .. 13 the byte offset (without the n
-// column), bits 14 and 15 an XOR on the n column, so that the builder's scattered stores fall in different
-// banks. Byte c / 5 of the block holds the column as digit c % 5, extracted at level 4 - c % 5.
-// DIAG: lane q decodes block q. Bytes 0 .. 23 four at a time, bytes 4u, 4u + 2 and 4u + 1, 4u + 3 in the
-// halves of an even and an odd register: step 5u + level, k slots 2q, 2q + 1 (even) and 2q + 8, 2q + 9
-// (odd); bytes 24 and 25 share a register whose levels fill steps 30 .. 32. The offset is without 8q.
-// Else: the four lanes share a block's first 24 bytes, six each, in steps 8 block .. 8 block + 7: the first
-// four as above in five steps, the last two as bytes 24 and 25 above in three. Bytes 24 and 25 of block q
-// go to lane q in steps 32 .. 34 (bit 13 set). The offset is without the block.
-template <bool DIAG>
-__device__ __forceinline__ uint32_t x_b_offset(int c) {
-  const int byte = c / 5, level = 4 - (c - 5 * byte);
-  const uint32_t half_step = (uint32_t)((level >> 1) * 256 + 4 * (level & 1)), xor_n = (uint32_t)(level & 3) << 14;
-  if (byte >= 24) return half_step + 2 * (byte - 24) + (DIAG ? 30 * 256 : 1u << 13);
-  const int w = DIAG ? byte & 3 : byte % 6;
-  const uint32_t base = DIAG ? (uint32_t)(byte >> 2) * 1280 : (uint32_t)(byte / 6) * 8;
-  if (w < 4) return (base + level * 256 + 4 * (w & 1) + 2 * (w >> 1)) | xor_n;
-  return base + 1280 + half_step + 2 * (w - 4);
-}
-
-// Sixteen columns of x (row m) and v per lane: columns 16 lane .. 16 lane + 15 of chunk ch, zero past K.
-struct XRow {
-  uint32_t x[8], v[8];
-};
-__device__ __forceinline__ void x_load_row(const XProblem& a, int ch, int m, int lane, XRow& r) {
-  const int col = ch * kXChunkCols + 16 * lane;
-  const uint16_t* x = a.x + (size_t)m * a.K + col;
-  const uint16_t* v = a.v + col;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) r.x[i] = r.v[i] = 0u;
-  if (a.xv_vec) {  // rows of whole 16-byte vectors, 16-byte aligned
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-      if (col + 8 * i < a.K) {
-        const uint4 t = __ldg(reinterpret_cast<const uint4*>(x) + i), w = __ldg(reinterpret_cast<const uint4*>(v) + i);
-        r.x[4 * i] = t.x; r.x[4 * i + 1] = t.y; r.x[4 * i + 2] = t.z; r.x[4 * i + 3] = t.w;
-        r.v[4 * i] = w.x; r.v[4 * i + 1] = w.y; r.v[4 * i + 2] = w.z; r.v[4 * i + 3] = w.w;
-      }
-  } else {
-#pragma unroll
-    for (int i = 0; i < 16; ++i)
-      if (col + i < a.K) {
-        r.x[i >> 1] |= (uint32_t)__ldg(x + i) << (16 * (i & 1));
-        r.v[i >> 1] |= (uint32_t)__ldg(v + i) << (16 * (i & 1));
-      }
-  }
-}
-
-// One batch row's B operand of a chunk, by one warp (lane = 16 columns; boff: the block's places, two
-// columns a word). DIAG (M =
-// 1): column pair q of the tile for block q, else column pair m % 4. The factor 2^-E and the blocks'
-// sums of x go to fold[m] and sx[block][m].
-template <bool DIAG>
-__device__ __forceinline__ void x_build_row(const XRow& r, int m, const uint32_t* boff, uint8_t* bt, float* fold,
-                                            float* sx, int lane) {
-  // v*x is exact in fp32; formed here for the largest and again below (sixteen registers fewer)
-  auto product = [&](int i) {
-    return h2f((uint16_t)(r.v[i >> 1] >> (16 * (i & 1)))) * h2f((uint16_t)(r.x[i >> 1] >> (16 * (i & 1))));
-  };
-  float sum = 0.f, lmax = 0.f, probe = 0.f;
-#pragma unroll
-  for (int i = 0; i < 16; ++i) {
-    const float p = product(i);
-    sum += h2f((uint16_t)(r.x[i >> 1] >> (16 * (i & 1))));
-    lmax = fmaxf(lmax, fabsf(p));
-    probe = fmaf(p, 0.f, probe);
-  }
-  // an infinity or NaN in v*x (fmaxf drops NaN) makes the row's result NaN
-  if (!(fabsf(probe) <= 1.f)) lmax = __int_as_float(0x7f800000);
-  const uint32_t amax = __reduce_max_sync(0xffffffffu, __float_as_uint(lmax));
-  const int e = amax ? (int)(amax >> 23) - 127 : 0;  // |v*x| < 2^(e + 1)
-  const float sc = __uint_as_float((uint32_t)(127 + 13 - e) << 23);  // half of 2^E, E = 14 - e
-  const int q = lane >> 3, n = DIAG ? 2 * q : 2 * (m & 3);  // the lane's block, the hi column
-  uint8_t* tile = bt + (DIAG ? 8 * q : (m >> 2) * kXBTileBytes + 2048 * q);
-  const int tail = 8192 - 2048 * q + 8 * q;  // from there: bytes 24 and 25
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const float f0 = product(2 * i) * sc, f1 = product(2 * i + 1) * sc;
-    const uint32_t ow = boff[8 * (lane & 7) + i];
-    const __half2 hi = __floats2half2_rn(f0, f1);
-    const __half2 lo = __floats2half2_rn(f0 - __low2float(hi), f1 - __high2float(hi));
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const uint32_t o = (ow >> (16 * k)) & 0xFFFFu;
-      const uint32_t lx = (uint32_t)n ^ (o >> 14);  // n even: the lo column n + 1 is n's neighbour XOR 1
-      uint8_t* d = tile + (DIAG ? o & 0x3FFFu : (o & 0x1FFFu) + (o & 0x2000u ? tail : 0));
-      *reinterpret_cast<__half*>(d + 32 * lx) = k ? __high2half(hi) : __low2half(hi);
-      *reinterpret_cast<__half*>(d + 32 * (lx ^ 1u)) = k ? __high2half(lo) : __low2half(lo);
-    }
-  }
-  sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-  sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-  sum += __shfl_xor_sync(0xffffffffu, sum, 4);
-  if ((lane & 7) == 0) sx[16 * q + m] = sum;
-  if (lane == 0) fold[m] = __uint_as_float((uint32_t)(127 - 14 + e) << 23);  // 2^-E
-}
-
-// The unit's scales as (alpha, beta) fp16 pairs [256 rows][4 blocks] (0 past the last block), by copies
-// where a row's four pairs are one aligned 16-byte vector.
-template <int H>
-__device__ __forceinline__ void x_stage_scales(const XProblem& a, const XPos& c, uint8_t* dst, int ht) {
-  const int nb = min(4, a.n_blocks - 4 * c.ch);
-#pragma unroll
-  for (int k = 0; k < kXTileRows / (32 * H); ++k) {
-    const int r = ht + k * 32 * H, row = c.t * kXTileRows + r;
-    if (row >= a.N) break;
-    if (a.scales_vec) {
-      x_cp16(smem_u32(dst + r * 16), a.scales + 2 * ((size_t)row * a.G + 4 * c.ch));
-      continue;
-    }
-    uint32_t w[4] = {0u, 0u, 0u, 0u};
-    if (a.G == 1) {
-      const uint32_t ab = (uint32_t)__ldg(a.scales + (size_t)row * (a.bias ? 2 : 1)) |
-                          (a.bias ? (uint32_t)__ldg(a.scales + (size_t)row * 2 + 1) << 16 : 0u);
-#pragma unroll
-      for (int b = 0; b < 4; ++b) w[b] = b < nb ? ab : 0u;
-    } else {
-#pragma unroll
-      for (int b = 0; b < 4; ++b)
-        if (b < nb) {
-          const size_t e = (size_t)row * a.G + 4 * c.ch + b;
-          w[b] = a.bias ? (uint32_t)__ldg(a.scales + 2 * e) | (uint32_t)__ldg(a.scales + 2 * e + 1) << 16
-                        : (uint32_t)__ldg(a.scales + e);
-        }
-    }
-    *reinterpret_cast<uint4*>(dst + r * 16) = make_uint4(w[0], w[1], w[2], w[3]);
-  }
-}
-
-// The unit's residual values as stored, 16 per (group of four rows, step) = (ht >> 1, ht & 1), zero past
-// the last entry: by copies where rows are whole aligned 8-byte words.
-__device__ __forceinline__ void x_stage_residual(const XProblem& a, const XPos& c, int st0, int n_steps, uint8_t* vals,
-                                                 int ht) {
-  const int gl = ht >> 1, k = ht & 1, grp = c.t * (kXTileRows / 4) + gl;
-  if (gl >= kXTileRows / 4 || k >= n_steps || 4 * grp >= a.N) return;
-  const int e0 = 16 * (st0 + k), ne = min(16, a.s - e0);
-  const size_t e = (size_t)grp * a.s + e0;
-  uint8_t* d = vals + gl * kXResStride + 32 * k;
-  if (a.res_vec) {
-    const uint8_t* src = reinterpret_cast<const uint8_t*>(a.rvals) + (a.fp8 ? e : 2 * e);
-    const int n = a.fp8 ? ne : 2 * ne;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-      if (i < 2 || !a.fp8) x_cp8(smem_u32(d + 8 * i), 8 * i < n ? src + 8 * i : src, 8 * i < n ? 8 : 0);
-    return;
-  }
-  for (int i = 0; i < 16; ++i) {
-    if (a.fp8) d[i] = i < ne ? __ldg(reinterpret_cast<const uint8_t*>(a.rvals) + e + i) : (uint8_t)0;
-    else reinterpret_cast<uint16_t*>(d)[i] = i < ne ? __ldg(reinterpret_cast<const uint16_t*>(a.rvals) + e + i) : (uint16_t)0;
-  }
-}
-
-// The position bytes of the same entries, in one word.
-__device__ __forceinline__ uint32_t x_load_pos(const XProblem& a, const XPos& c, int st0, int n_steps, int ht) {
-  const int k = ht & 1, grp = c.t * (kXTileRows / 4) + (ht >> 1);
-  uint32_t w = 0u;
-  if (ht < kXTileRows / 2 && k < n_steps && 4 * grp < a.N) {
-    const int rs = (a.s + 3) >> 2, b0 = 4 * (st0 + k);
-    const uint8_t* pp = a.ridx + (size_t)grp * rs + b0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-      if (b0 + i < rs) w |= (uint32_t)__ldg(pp + i) << (8 * i);
-  }
-  return w;
-}
-
-// The unit's salient column of this lane's entry (-1: none).
-__device__ __forceinline__ int x_load_sal(const XProblem& a, int st0, int n_steps, int lane) {
-  const int e = 16 * st0 + lane;
-  if (lane >= 16 * n_steps || e >= a.s) return -1;
-  const int col = __ldg(a.sal + e);
-  return col < 0 ? 0 : (col >= a.K ? a.K - 1 : col);
-}
-
-// ---------------------------------------------------------------- consumers
-
-// Two FP8 E4M3 bytes as an fp16 pair (exact).
-__device__ __forceinline__ uint32_t x_e4m3x2(uint32_t b) {
-  uint32_t d;
-  asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(d) : "h"((uint16_t)b));
-  return d;
-}
-
-// One residual step: A = the row's values at the entries whose stored position is the row.
-template <int MT, int BLK>
-__device__ __forceinline__ void x_res_step(const uint8_t* vals, const uint8_t* pos, const uint8_t* rb, int step, bool fp8,
-                                           int tr, int g, int q, int lane, float (&acc)[BLK][MT][4]) {
-  uint2 b[MT];
-#pragma unroll
-  for (int j = 0; j < MT; ++j) b[j] = *reinterpret_cast<const uint2*>(rb + j * kXResBBytes + (step * 32 + lane) * 8);
-#pragma unroll
-  for (int k = 0; k < BLK; ++k) {
-    uint32_t av[4];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int gl = (tr + 16 * k + 8 * h + g) >> 2;
-      uint32_t lo, hi;
-      if (fp8) {
-        const uint32_t w = *reinterpret_cast<const uint32_t*>(vals + gl * kXResStride + 32 * step + 4 * q);
-        lo = x_e4m3x2(w & 0xFFFFu);
-        hi = x_e4m3x2(w >> 16);
-      } else {
-        const uint2 w = *reinterpret_cast<const uint2*>(vals + gl * kXResStride + 32 * step + 8 * q);
-        lo = w.x;
-        hi = w.y;
-      }
-      // two-bit fields of d are zero where the entry is stored at this row's position
-      const uint32_t d = (uint32_t)pos[gl * 8 + 4 * step + q] ^ ((uint32_t)(g & 3) * 0x55u);
-      const uint32_t nz = d | (d >> 1);
-      const uint32_t k0 = ((nz & 1u) - 1u) & 0x0000ffffu, k1 = (((nz >> 2) & 1u) - 1u) & 0xffff0000u;
-      const uint32_t k2 = (((nz >> 4) & 1u) - 1u) & 0x0000ffffu, k3 = (((nz >> 6) & 1u) - 1u) & 0xffff0000u;
-      av[h] = lo & (k0 | k1);
-      av[2 + h] = hi & (k2 | k3);
-    }
-#pragma unroll
-    for (int j = 0; j < MT; ++j) x_mma(acc[k][j], av[0], av[1], av[2], av[3], b[j]);
-  }
-}
-
-// A pair of code bytes decoded digit by digit, the highest first (see the header). IMAD: the digits are
-// taken out for the next step as r - (r & 0xC000C000) = r + digit() - 0xC000C000 on the multiply pipe
-// instead of a mask on the logic pipe, which is the busier one: with every other register that way the
-// decode alone runs at 50.7 weights per clock per SM against 47.9.
-template <bool IMAD>
-struct XDigits {
-  uint32_t r;
-  __device__ __forceinline__ void start(uint32_t bytes) { r = bytes * 203u; }  // a byte in each half
-  __device__ __forceinline__ uint32_t digit() const { return ~r & 0xC000C000u; }
-  __device__ __forceinline__ void next() {
-    if (IMAD) {
-      uint32_t t;
-      asm("mad.lo.u32 %0, %1, 3, %2;" : "=r"(t) : "r"(digit()), "r"(0u - 3u * 0xC000C000u));
-      asm("mad.lo.u32 %0, %1, 3, %2;" : "=r"(r) : "r"(r), "r"(t));
-    } else {
-      r = (r & 0x3FFF3FFFu) * 3u;
-    }
-  }
-};
-
-// M = 1: the unit's 33 steps for the warp's 16-row blocks, lane q's weights all of block q. codes: the
-// stage's rows, from the aligned word that holds the lane's first byte; sh: 0, or 16 when that byte is the
-// word's third. sum[.][0 / 1]: rows g, g + 8 over block q. (2T leaves 11-bit products, which the tensor
-// core's sums lose little of; alpha in A would make them 22 bits, truncated at every step: 6.7e-7.)
-template <int BLK>
-__device__ __forceinline__ void x_decode_diag(const uint8_t* codes, int row_slot, int sh, const uint8_t* bt, int lane,
-                                              float (&sum)[BLK][2]) {
-  constexpr int R = 2 * BLK;  // the thread's rows: 8 apart
-  const int stride = 8 * row_slot;
-  float acc[BLK][4];
-#pragma unroll
-  for (int k = 0; k < BLK; ++k) acc[k][0] = acc[k][1] = acc[k][2] = acc[k][3] = 0.f;
-  uint32_t w[R];
-#pragma unroll
-  for (int r = 0; r < R; ++r) w[r] = *reinterpret_cast<const uint32_t*>(codes + r * stride);
-#pragma unroll 2
-  for (int u = 0; u < 6; ++u) {
-    XDigits<false> e[R];
-    XDigits<true> o[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const uint32_t nx = *reinterpret_cast<const uint32_t*>(codes + r * stride + 4 * u + 4);
-      const uint32_t x = __funnelshift_r(w[r], nx, sh);
-      w[r] = nx;
-      e[r].start(x & 0x00FF00FFu);
-      o[r].start(__byte_perm(x, 0u, 0x4341));
-    }
-#pragma unroll
-    for (int l = 0; l < 5; ++l) {
-      const uint2 b = *reinterpret_cast<const uint2*>(bt + (5 * u + l) * 256 + (lane ^ (4 * (l & 3))) * 8);
-#pragma unroll
-      for (int k = 0; k < BLK; ++k)
-        x_mma(acc[k], e[2 * k].digit(), e[2 * k + 1].digit(), o[2 * k].digit(), o[2 * k + 1].digit(), b);
-      if (l < 4) {
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-          e[r].next();
-          o[r].next();
-        }
-      }
-    }
-  }
-  XDigits<false> e[R];
-#pragma unroll
-  for (int r = 0; r < R; ++r) e[r].start(__byte_perm(w[r] >> sh, 0u, 0x4140));
-#pragma unroll
-  for (int l = 0; l < 5; l += 2) {
-    const uint2 b = *reinterpret_cast<const uint2*>(bt + ((30 + l / 2) * 32 + lane) * 8);
-    uint32_t a0[R], a1[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      a0[r] = e[r].digit();
-      e[r].next();
-      a1[r] = l < 4 ? e[r].digit() : 0u;
-      e[r].next();
-    }
-#pragma unroll
-    for (int k = 0; k < BLK; ++k) x_mma(acc[k], a0[2 * k], a0[2 * k + 1], a1[2 * k], a1[2 * k + 1], b);
-  }
-#pragma unroll
-  for (int k = 0; k < BLK; ++k) {
-    sum[k][0] = acc[k][0] + acc[k][1];
-    sum[k][1] = acc[k][2] + acc[k][3];
-  }
-}
-
-// M >= 2: the unit's 35 steps. The four lanes share each block (six bytes each, one accumulation of eight
-// steps, scaled by the rows' alpha in fp32: run += alpha_b 2^-E sum + beta_b sum_b(x)); the blocks' last
-// two bytes go to one lane each and carry alpha in A (a sixteenth of the columns, three steps). row: the
-// offset of the thread's first row in the stage; off: of the unit in the row.
-template <int MT, int BLK>
-__device__ __forceinline__ void x_decode_rows(const uint8_t* row, int off, int row_slot, const uint8_t* bt,
-                                              const uint8_t* sc, const float* fold, const float* sx, bool bias,
-                                              int q, int lane, float (&run)[BLK][MT][2]) {
-  constexpr int R = 2 * BLK;
-  const int stride = 8 * row_slot;
-  // the unit's sum on its own before it joins the tile's: 28 additions in a row instead of 112 for K = 14336
-  float acc[BLK][MT][4], part[BLK][MT][2];
-#pragma unroll
-  for (int k = 0; k < BLK; ++k)
-#pragma unroll
-    for (int j = 0; j < MT; ++j) part[k][j][0] = part[k][j][1] = 0.f;
-#pragma unroll 1
-  for (int blk = 0; blk < 4; ++blk) {
-    const int o0 = off + 26 * blk + 6 * q, sh = 8 * (o0 & 2);
-    const uint8_t* wp = row + (o0 & ~3);
-    const uint8_t* bb = bt + blk * 2048;
-    XDigits<false> e[R], y[R];
-    XDigits<true> o[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const uint32_t w0 = *reinterpret_cast<const uint32_t*>(wp + r * stride);
-      const uint32_t w1 = *reinterpret_cast<const uint32_t*>(wp + r * stride + 4);
-      const uint32_t x = __funnelshift_r(w0, w1, sh);
-      e[r].start(x & 0x00FF00FFu);
-      o[r].start(__byte_perm(x, 0u, 0x4341));
-      y[r].start(__byte_perm(w1 >> sh, 0u, 0x4140));
-    }
-#pragma unroll
-    for (int l = 0; l < 5; ++l) {
-      uint2 b[MT];
-#pragma unroll
-      for (int j = 0; j < MT; ++j)
-        b[j] = *reinterpret_cast<const uint2*>(bb + j * kXBTileBytes + l * 256 + (lane ^ (4 * (l & 3))) * 8);
-#pragma unroll
-      for (int k = 0; k < BLK; ++k) {
-        const uint32_t a0 = e[2 * k].digit(), a1 = e[2 * k + 1].digit(), a2 = o[2 * k].digit(), a3 = o[2 * k + 1].digit();
-#pragma unroll
-        for (int j = 0; j < MT; ++j) {
-          if (l == 0) x_mma_first(acc[k][j], a0, a1, a2, a3, b[j]);
-          else x_mma(acc[k][j], a0, a1, a2, a3, b[j]);
-        }
-      }
-      if (l < 4) {
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-          e[r].next();
-          o[r].next();
-        }
-      }
-    }
-#pragma unroll
-    for (int l = 0; l < 5; l += 2) {
-      uint2 b[MT];
-#pragma unroll
-      for (int j = 0; j < MT; ++j)
-        b[j] = *reinterpret_cast<const uint2*>(bb + j * kXBTileBytes + (5 + l / 2) * 256 + lane * 8);
-      uint32_t a0[R], a1[R];
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        a0[r] = y[r].digit();
-        y[r].next();
-        a1[r] = l < 4 ? y[r].digit() : 0u;
-        y[r].next();
-      }
-#pragma unroll
-      for (int k = 0; k < BLK; ++k)
-#pragma unroll
-        for (int j = 0; j < MT; ++j) x_mma(acc[k][j], a0[2 * k], a0[2 * k + 1], a1[2 * k], a1[2 * k + 1], b[j]);
-    }
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const uint32_t ab = *reinterpret_cast<const uint32_t*>(sc + r * 128 + 4 * blk);
-      const float al = h2f((uint16_t)ab), be = h2f((uint16_t)(ab >> 16));
-#pragma unroll
-      for (int j = 0; j < MT; ++j) {
-        float& t = part[r >> 1][j][r & 1];
-        const float* a2 = &acc[r >> 1][j][2 * (r & 1)];
-        t = fmaf(al, (a2[0] + a2[1]) * fold[4 * j + q], t);
-        if (bias) t = fmaf(be, sx[16 * blk + 4 * j + q], t);
-      }
-    }
-  }
-  // bytes 24 and 25 of block q; alpha * 2T must stay finite: rows with some |alpha| >= 2^14 take alpha / 4
-  uint32_t al[R];
-  bool big = false;
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    al[r] = __byte_perm(*reinterpret_cast<const uint32_t*>(sc + r * 128 + 4 * q), 0u, 0x1010);
-    big = big || (al[r] & 0x7FFFu) >= 0x7400u;
-  }
-  float up = 1.f;
-  if (__any_sync(0xffffffffu, big)) {
-    up = 4.f;
-#pragma unroll
-    for (int r = 0; r < R; ++r) al[r] = x_hmul2(al[r], 0x34003400u);
-  }
-  XDigits<false> y[R];
-  const int o0 = off + 26 * q + 24;
-#pragma unroll
-  for (int r = 0; r < R; ++r)
-    y[r].start(__byte_perm((uint32_t)*reinterpret_cast<const uint16_t*>(row + o0 + r * stride), 0u, 0x4140));
-#pragma unroll
-  for (int l = 0; l < 5; l += 2) {
-    uint2 b[MT];
-#pragma unroll
-    for (int j = 0; j < MT; ++j)
-      b[j] = *reinterpret_cast<const uint2*>(bt + j * kXBTileBytes + (32 + l / 2) * 256 + lane * 8);
-    uint32_t a0[R], a1[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      a0[r] = x_hmul2(y[r].digit(), al[r]);
-      y[r].next();
-      a1[r] = l < 4 ? x_hmul2(y[r].digit(), al[r]) : 0u;
-      y[r].next();
-    }
-#pragma unroll
-    for (int k = 0; k < BLK; ++k)
-#pragma unroll
-      for (int j = 0; j < MT; ++j) {
-        if (l == 0) x_mma_first(acc[k][j], a0[2 * k], a0[2 * k + 1], a1[2 * k], a1[2 * k + 1], b[j]);
-        else x_mma(acc[k][j], a0[2 * k], a0[2 * k + 1], a1[2 * k], a1[2 * k + 1], b[j]);
-      }
-  }
-#pragma unroll
-  for (int k = 0; k < BLK; ++k)
-#pragma unroll
-    for (int j = 0; j < MT; ++j) {
-      const float F = fold[4 * j + q] * up;
-      run[k][j][0] += fmaf(acc[k][j][0] + acc[k][j][1], F, part[k][j][0]);
-      run[k][j][1] += fmaf(acc[k][j][2] + acc[k][j][3], F, part[k][j][1]);
-    }
-}
-
-// MT: n8 tiles (four batch rows each). DIAG: M = 1, column pairs by lane (see the header); MT = 1 then.
-template <int MT, bool DIAG>
-__global__ void __launch_bounds__(x_threads(MT), 1) qtea_gemv_b3mma_kernel(const __grid_constant__ TensorMaps maps, const __grid_constant__ XParams P) {
-  // SETS sets of H helper warps take units in turn; CW consumer warps of BLK 16-row blocks
-  constexpr int H = kXHelpers, SETS = x_sets(MT), BLK = x_blocks(MT), CW = kXTileRows / 16 / BLK;
-  constexpr int kXThreads = x_threads(MT), kXHelperThreads = 32 * H;
-  extern __shared__ __align__(128) uint8_t smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int u0 = P.cta_u0[blockIdx.x], u1 = P.cta_u0[blockIdx.x + 1], n_units = u1 - u0;
-  const int S = P.n_stages, row_slot = P.row_slot, NP = P.n_problems, M = P.M;
-  const XStage lay = x_stage_layout(MT, row_slot);
-  XProblem* tab = reinterpret_cast<XProblem*>(smem + (size_t)S * lay.total);
-  uint64_t* full = reinterpret_cast<uint64_t*>(tab + kMaxProblems);  // [S] the helpers' copies and stores landed
-  uint64_t* empty = full + S;                                        // [S] consumers released it
-  uint32_t* boff = reinterpret_cast<uint32_t*>(empty + S);           // [64] x_b_offset of two columns each
-  {
-    const uint32_t* src = reinterpret_cast<const uint32_t*>(P.prob);
-    uint32_t* dst = reinterpret_cast<uint32_t*>(tab);
-    for (int i = threadIdx.x; i < NP * (int)(sizeof(XProblem) / 4); i += kXThreads) dst[i] = src[i];
-  }
-  if (threadIdx.x < 64) boff[threadIdx.x] = x_b_offset<DIAG>(2 * threadIdx.x) | x_b_offset<DIAG>(2 * threadIdx.x + 1) << 16;
-  // B columns that no batch row (or, with DIAG, no lane's block) writes, and k slots of pad digits, stay
-  // zero in every stage; the scales of rows past N too
-  for (int s = 0; s < S; ++s) {
-    uint4* z = reinterpret_cast<uint4*>(smem + (size_t)s * lay.total + lay.scales);
-    for (int i = threadIdx.x; i < (lay.b_end - lay.scales) / 16; i += kXThreads) z[i] = make_uint4(0u, 0u, 0u, 0u);
-  }
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < S; ++i) {
-      mbar_init(smem_u32(&full[i]), 2 * kXHelperThreads + (P.tma ? 1 : 0));  // a thread's copies, its stores; the TMA
-      mbar_init(smem_u32(&empty[i]), CW);
-    }
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  __syncthreads();
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-
-  if (warp < SETS * H) {
-    // ---------------------------------------------------------------- helpers
-    const int set = warp / H, hw = warp - set * H, ht = threadIdx.x - set * kXHelperThreads;
-    const uint64_t pol = l2_evict_first_policy();
-    auto advance = [&](XPos& d) {
-#pragma unroll
-      for (int k = 0; k < SETS; ++k) x_next(d, tab);
-    };
-    XPos c = x_pos(tab, NP, u0);
-    for (int k = 0; k < set; ++k) x_next(c, tab);
-    // a unit's codes: one TMA box where rows are whole 16-byte vectors, else copies by every helper thread
-    const bool tma = P.tma != 0;
-    auto issue_codes = [&](const XPos& d, int st) {
-      uint8_t* sb = smem + (size_t)st * lay.total;
-      if (!tma) {
-        x_issue_codes<H>(tab[d.p], d, smem_u32(sb), row_slot, ht);
-      } else if (ht == 0) {
-        const uint32_t bar = smem_u32(&full[st]);
-        mbar_arrive_expect_tx(bar, kXTileRows * kXBoxBytes);
-        tma_load_2d_hint(smem_u32(sb), &maps.m[d.p], (d.ch * kXChunkBytes) & ~15, d.t * kXTileRows, bar, pol);
-      }
-    };
-    {
-      // the codes belong to the library and no kernel writes them: the first stages' copies start
-      // before the grid dependency wait
-      XPos f = c;
-      for (int i = set; i < S && i < n_units; i += SETS) {
-        issue_codes(f, i);
-        advance(f);
-      }
-    }
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    // a unit's loads to registers go out a unit ahead: x and v of the warp's first batch row, the
-    // positions, and x at the salient columns (their indices another unit ahead)
-    XRow row;
-    uint32_t pos = 0u;
-    uint16_t xs = 0;
-    int col = -1, col_next = -1;
-    XPos n1 = c;  // the set's unit after c
-    auto load_ahead = [&](const XPos& d) {  // d's loads; col holds its salient columns
-      const XProblem& a = tab[d.p];
-      const int rsn = x_res_steps(d, a);
-      if (hw < M) x_load_row(a, d.ch, hw, lane, row);
-      pos = x_load_pos(a, d, d.rs, rsn, ht);
-      xs = hw < M && col >= 0 ? __ldg(a.x + (size_t)hw * a.K + col) : (uint16_t)0;
-    };
-    if (set < n_units) {
-      col = x_load_sal(tab[c.p], c.rs, x_res_steps(c, tab[c.p]), lane);
-      load_ahead(c);
-    }
-    for (int i = set; i < n_units; i += SETS) {
-      const int st = i % S;
-      uint8_t* sb = smem + (size_t)st * lay.total;
-      const XProblem& a = tab[c.p];
-      const int rsn = x_res_steps(c, a);
-      if (i + SETS < n_units) advance(n1);
-      col_next = i + SETS < n_units ? x_load_sal(tab[n1.p], n1.rs, x_res_steps(n1, tab[n1.p]), lane) : -1;
-      if (i >= S) {
-        if (!mbar_wait(smem_u32(&empty[st]), (uint32_t)((i / S - 1) & 1), P.status)) break;
-        issue_codes(c, st);
-      }
-      x_stage_scales<H>(a, c, sb + lay.scales, ht);
-      if (rsn > 0) {
-        x_stage_residual(a, c, c.rs, rsn, sb + lay.rvals, ht);
-        if (ht < kXTileRows / 2) *reinterpret_cast<uint32_t*>(sb + lay.rpos + 4 * ht) = pos;
-      }
-      x_cp_arrive(smem_u32(&full[st]));
-      for (int m = hw; m < M; m += H) {
-        if (m > hw) {
-          x_load_row(a, c.ch, m, lane, row);
-          xs = col >= 0 ? __ldg(a.x + (size_t)m * a.K + col) : (uint16_t)0;
-        }
-        if (lane < 16 * rsn)  // x at the salient entries: the hi column of the row's pair
-          *reinterpret_cast<uint16_t*>(sb + lay.rb + (m >> 2) * kXResBBytes +
-                                       ((lane >> 4) * 32 + 8 * (m & 3) + ((lane >> 2) & 3)) * 8 + 2 * (lane & 3)) = xs;
-        x_build_row<DIAG>(row, m, boff, sb + lay.b, reinterpret_cast<float*>(sb + lay.fold),
-                          reinterpret_cast<float*>(sb + lay.sx), lane);
-      }
-      mbar_arrive(smem_u32(&full[st]));
-      c = n1;
-      col = col_next;
-      if (i + SETS < n_units) load_ahead(c);
-    }
-    asm volatile("cp.async.wait_all;" ::: "memory");  // no copy in flight when the CTA exits
-    if (tma && ht == 0)
-      for (int j = n_units < S ? 0 : n_units - S; j < n_units; ++j)
-        if (j % SETS == set && !mbar_wait(smem_u32(&full[j % S]), (uint32_t)((j / S) & 1), P.status)) break;
-    return;
-  }
-
-  // ---------------------------------------------------------------- consumers
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  const int g = lane >> 2, q = lane & 3, tr = (warp - SETS * H) * 16 * BLK;
-  const int ct = threadIdx.x - SETS * kXHelperThreads;
-  float run[BLK][MT][2];  // [row block][tile][row g or g + 8]: batch row 4 tile + q (DIAG: block q's share)
-#pragma unroll
-  for (int k = 0; k < BLK; ++k)
-#pragma unroll
-    for (int j = 0; j < MT; ++j) run[k][j][0] = run[k][j][1] = 0.f;
-  XPos c = x_pos(tab, NP, u0);
-  for (int i = 0; i < n_units; ++i) {
-    const int st = i % S;
-    const uint8_t* sb = smem + (size_t)st * lay.total;
-    const XProblem& a = tab[c.p];
-    const uint32_t par = (uint32_t)((i / S) & 1);
-    if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&full[st]), par, P.status))) break;
-    const int rsn = x_res_steps(c, a);
-    if (rsn > 0) {
-      float acc[BLK][MT][4];
-#pragma unroll
-      for (int k = 0; k < BLK; ++k)
-#pragma unroll
-        for (int j = 0; j < MT; ++j)
-#pragma unroll
-          for (int z = 0; z < 4; ++z) acc[k][j][z] = 0.f;
-      for (int s = 0; s < rsn; ++s)
-        x_res_step<MT, BLK>(sb + lay.rvals, sb + lay.rpos, sb + lay.rb, s, a.fp8 != 0, tr, g, q, lane, acc);
-#pragma unroll
-      for (int k = 0; k < BLK; ++k)
-#pragma unroll
-        for (int j = 0; j < MT; ++j) {
-          run[k][j][0] += acc[k][j][0];
-          run[k][j][1] += acc[k][j][2];
-        }
-    }
-    const uint8_t* sc = sb + lay.scales + (tr + g) * 16;
-    const float* fold = reinterpret_cast<const float*>(sb + lay.fold);
-    const float* sx = reinterpret_cast<const float*>(sb + lay.sx);
-    const int off = (int)(((size_t)(tr + g) * a.row_bytes + (size_t)c.ch * kXChunkBytes) & 15);
-    const uint8_t* row = sb + (tr + g) * row_slot;
-    if constexpr (DIAG) {
-      // the lane's block: 2^-E, alpha, and beta times its sum of x
-      const int o0 = off + 26 * q;
-      float sum[BLK][2];
-      x_decode_diag<BLK>(row + (o0 & ~3), row_slot, 8 * (o0 & 2), sb + lay.b, lane, sum);
-      const float F = fold[0], bx = sx[16 * q];
-#pragma unroll
-      for (int r = 0; r < 2 * BLK; ++r) {
-        const uint32_t ab = *reinterpret_cast<const uint32_t*>(sc + r * 128 + 4 * q);
-        run[r >> 1][0][r & 1] += fmaf(h2f((uint16_t)ab), sum[r >> 1][r & 1] * F, h2f((uint16_t)(ab >> 16)) * bx);
-      }
-    } else {
-      x_decode_rows<MT, BLK>(row, off, row_slot, sb + lay.b, sc, fold, sx, a.bias != 0, q, lane, run);
-    }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(smem_u32(&empty[st]));
-
-    if (c.ch == a.n_chunks - 1 || i == n_units - 1) {
-      // ---- the tile's epilogue once this CTA's part of it is done
-      if (DIAG) {  // the four blocks' shares, in lane order
-#pragma unroll
-        for (int k = 0; k < BLK; ++k)
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            run[k][0][h] += __shfl_xor_sync(0xffffffffu, run[k][0][h], 1);
-            run[k][0][h] += __shfl_xor_sync(0xffffffffu, run[k][0][h], 2);
-          }
-      }
-      const int A = a.unit_begin + c.t * a.n_chunks, B = A + a.n_chunks;
-      bool write = true;
-      if (A < u0) {
-        // not the first contributor: this CTA's partial rows, word by word (slot of this CTA)
-        uint32_t* mine = a.part + (size_t)blockIdx.x * 4 * MT * 256 + ct;
-#pragma unroll
-        for (int k = 0; k < BLK; ++k)
-#pragma unroll
-          for (int j = 0; j < MT; ++j)
-#pragma unroll
-            for (int h = 0; h < 2; ++h)
-              if (!DIAG || q == 0)
-                x_part_store(mine + ((k * MT + j) * 2 + h) * (32 * CW), __float_as_uint(run[k][j][h]) ^ kXPartEmpty);
-        write = false;
-      } else if (B > u1) {
-        // first contributor of a split tile: the partners' partial rows in CTA order, emptied again
-        const int last = x_unit_owner(B - 1, P.total_units, gridDim.x);
-        bool timed_out = false;
-        for (int cb = (int)blockIdx.x + 1; cb <= last; ++cb) {
-          uint32_t* src = a.part + (size_t)cb * 4 * MT * 256 + ct;
-          if (!DIAG || q == 0) {
-            uint32_t w[BLK * MT * 2];
-#pragma unroll
-            for (int z = 0; z < BLK * MT * 2; ++z) w[z] = x_part_load(src + z * (32 * CW));
-#pragma unroll
-            for (int z = 0; z < BLK * MT * 2; ++z) {
-              if (!timed_out && w[z] == 0u) {
-                const unsigned long long t0 = global_ns();
-                do {
-                  w[z] = x_part_load(src + z * (32 * CW));
-                  if (global_ns() - t0 > kWaitLimitNs) {
-                    atomicExch(P.status, (int)QTEA_ERR_TIMEOUT);
-                    timed_out = true;
-                    break;
-                  }
-                } while (w[z] == 0u);
-              }
-              run[z / (2 * MT)][(z / 2) % MT][z & 1] += __uint_as_float(w[z] ^ kXPartEmpty);
-              x_part_store(src + z * (32 * CW), 0u);
-            }
-          }
-        }
-      }
-      if (write) {
-#pragma unroll
-        for (int k = 0; k < BLK; ++k)
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int row = c.t * kXTileRows + tr + 16 * k + 8 * h + g;
-#pragma unroll
-            for (int j = 0; j < MT; ++j) {
-              const int m = DIAG ? 0 : 4 * j + q;
-              if (row < a.N && m < M && (!DIAG || q == 0)) a.y[(size_t)m * a.N + row] = run[k][j][h];
-            }
-          }
-      }
-#pragma unroll
-      for (int k = 0; k < BLK; ++k)
-#pragma unroll
-        for (int j = 0; j < MT; ++j) run[k][j][0] = run[k][j][1] = 0.f;
-    }
-    x_next(c, tab);
-  }
-}
-
-template <int MT, bool DIAG>
-cudaError_t x_set(size_t smem_optin) {
-  return cudaFuncSetAttribute(qtea_gemv_b3mma_kernel<MT, DIAG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)smem_optin);
-}
-
-}  // namespace
 
 cudaError_t b3mma_configure(size_t smem_optin) {
-  cudaError_t e = x_set<1, true>(smem_optin);
-  if (e == cudaSuccess) e = x_set<1, false>(smem_optin);
-  if (e == cudaSuccess) e = x_set<2, false>(smem_optin);
-  if (e == cudaSuccess) e = x_set<3, false>(smem_optin);
-  if (e == cudaSuccess) e = x_set<4, false>(smem_optin);
+  cudaError_t e = x_configure<1, kXDiag, true>(smem_optin);
+  if (e == cudaSuccess) e = x_configure<1, kXRows, true>(smem_optin);
+  if (e == cudaSuccess) e = x_configure<2, kXRows, true>(smem_optin);
+  if (e == cudaSuccess) e = x_configure<3, kXRows, true>(smem_optin);
+  if (e == cudaSuccess) e = x_configure<4, kXRows, true>(smem_optin);
   return e;
 }
 
 cudaError_t launch_b3mma(const TensorMaps& maps, const XParams& p, int grid, size_t smem, cudaStream_t st) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3((unsigned)x_threads(x_mt(p.M)));
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (p.M == 1) return cudaLaunchKernelEx(&cfg, qtea_gemv_b3mma_kernel<1, true>, maps, p);
-  switch (x_mt(p.M)) {
-    case 1: return cudaLaunchKernelEx(&cfg, qtea_gemv_b3mma_kernel<1, false>, maps, p);
-    case 2: return cudaLaunchKernelEx(&cfg, qtea_gemv_b3mma_kernel<2, false>, maps, p);
-    case 3: return cudaLaunchKernelEx(&cfg, qtea_gemv_b3mma_kernel<3, false>, maps, p);
-    default: return cudaLaunchKernelEx(&cfg, qtea_gemv_b3mma_kernel<4, false>, maps, p);
+  if (p.M == 1) return x_launch<1, kXDiag, true>(maps, p, grid, smem, st);
+  switch (x_mt(x_mode(true, p.M), p.M)) {
+    case 1: return x_launch<1, kXRows, true>(maps, p, grid, smem, st);
+    case 2: return x_launch<2, kXRows, true>(maps, p, grid, smem, st);
+    case 3: return x_launch<3, kXRows, true>(maps, p, grid, smem, st);
+    default: return x_launch<4, kXRows, true>(maps, p, grid, smem, st);
   }
 }
 

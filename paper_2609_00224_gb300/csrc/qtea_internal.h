@@ -353,47 +353,50 @@ struct LutParams {
 cudaError_t lut_configure(size_t smem_optin);
 cudaError_t launch_lut(const LutParams& p, bool grouped, int grid, cudaStream_t st);
 
-// ---------------------------------------------------------------- tensor-core base-3 kernel (any M)
-// See qtea_gemv_b3mma.cu. A unit is 256 rows x 512 columns; one stage of shared memory holds a unit's
-// code bytes (rows of row_slot bytes), its scales, its B operand and its share of the residual.
+// ---------------------------------------------------------------- tensor-core kernel with staged B operands
+// See qtea_mma.h: base-3 codes at any M, 2-bit codes at M >= 2 (at M = 1 with FP8 residual values). A unit is
+// 256 rows x 512 columns; one stage of shared memory holds a unit's code bytes (rows of row_slot bytes), its
+// scales, its B operand and its share of the residual.
 constexpr int kXTileRows = 256;
-constexpr int kXChunkCols = 512, kXChunkBytes = 104;           // four 128-column blocks of 26 bytes
-constexpr int kXBoxBytes = 112;                                // a row's part of a TMA box
-constexpr int kXSteps = 35;                                    // MMA steps of a unit (33 at M = 1)
-constexpr int kXBTileBytes = kXSteps * 32 * 8;                 // B of four batch rows (one n8 tile)
+constexpr int kXChunkCols = 512, kXChunkBytes = 104;           // four 128-column blocks (of 26 base-3 bytes)
+constexpr int kXBoxBytes = 112;                                // a base-3 row's part of a TMA box
+constexpr int kXSteps = 35;                                    // MMA steps of a base-3 unit (33 at M = 1)
+constexpr int kXBTileBytes = kXSteps * 32 * 8;                 // B of one n8 tile
+constexpr int kXTile2Bytes = 32 * 32 * 8;                      // the same for 2-bit codes: 32 steps
 constexpr int kXMaxStages = 4;
 constexpr int kXMaxChunks = 16384;                             // of a layout
 constexpr int kXResSteps = 2;                                  // residual steps (16 entries) a unit may take
 constexpr int kXResBBytes = kXResSteps * 32 * 8;               // their B per tile
 constexpr int kXResStride = 32 * kXResSteps + 8;               // their values per group of four rows
-__host__ __device__ constexpr int x_mt(int M) { return (M + 3) / 4; }
 constexpr int kXHelpers = 4;                                   // warps of a helper set
-__host__ __device__ constexpr int x_sets(int mt) { return 2; }
-__host__ __device__ constexpr int x_blocks(int mt) { return 2; }   // 16-row blocks of a consumer warp
-__host__ __device__ constexpr int x_threads(int mt) {
-  return 32 * (kXTileRows / 16 / x_blocks(mt) + x_sets(mt) * kXHelpers);
-}
-
+constexpr int kXBlocks = 2;                                    // 16-row blocks of a consumer warp
+constexpr int kXSets = 2;                                      // helper sets
+constexpr int kXThreads = 32 * (kXTileRows / 16 / kXBlocks + kXSets * kXHelpers);
+// Forms (XMode in qtea_mma.h) and n8 tiles.
+__host__ __device__ constexpr int x_mode(bool base3, int M) { return base3 ? (M == 1 ? 0 : 1) : (M <= 4 ? 2 : 3); }
+__host__ __device__ constexpr int x_mt(int mode, int M) { return mode == 3 ? (M + 7) / 8 : (M + 3) / 4; }
 struct XStage {  // byte offsets within a stage; the codes start it
-  int scales, rvals, rpos, b, rb, fold, sx, b_end, total;
+  int scales, rvals, rpos, b, rb, v, fold, sx, b_end, total;
 };
-__host__ __device__ inline XStage x_stage_layout(int mt, int row_slot) {
+__host__ __device__ inline XStage x_stage_layout(int mode, int mt, int row_slot) {
   XStage o;
   o.scales = kXTileRows * row_slot;
   o.rvals = o.scales + kXTileRows * 16;
   o.rpos = o.rvals + kXTileRows / 4 * kXResStride;
   o.b = o.rpos + kXTileRows / 4 * 4 * kXResSteps;
-  o.rb = o.b + mt * kXBTileBytes;
-  o.fold = o.rb + mt * kXResBBytes;       // [16] floats
+  o.rb = o.b + mt * (mode <= 1 ? kXBTileBytes : kXTile2Bytes);
+  o.v = o.rb + mt * kXResBBytes;
+  o.fold = o.v + (mode == 3 ? 1024 : 0);  // [16] floats
   o.sx = o.fold + 64;                     // [4 blocks][16] floats
   o.b_end = o.sx + 256;
-  o.total = (o.b_end + 127) / 128 * 128;
+  const int unit = mode <= 1 ? 128 : 1024;  // 1024: the 128-byte swizzle of 2-bit codes
+  o.total = (o.b_end + unit - 1) / unit * unit;
   return o;
 }
 
 struct XProblem {
   const uint16_t* x;        // [M][K]
-  const uint8_t* packed;    // [N][row_bytes] base-3
+  const uint8_t* packed;    // [N][row_bytes] (base-3 rows without a tensor map)
   const uint16_t* scales;   // [N][G] alpha, or [N][G][2] (alpha, beta) with bias
   const uint16_t* v;        // [K]
   const int32_t* sal;       // [s]
@@ -403,7 +406,7 @@ struct XProblem {
   uint32_t* part;           // [grid][4 MT][256] partial rows of split tiles, zero between calls
   int N, K, s, row_bytes, n_blocks, n_tiles, n_chunks;
   int fp8, G, bias;         // G: scale groups per row (1, or one per block)
-  int scales_vec;           // a row's four (alpha, beta) pairs of a chunk are one aligned 16-byte vector
+  int scales_vec;           // a row's four (alpha, beta) pairs of a chunk are one aligned 16-byte vector (alphas: 8)
   int xv_vec;               // rows of x, and v, are whole, aligned 16-byte vectors
   int res_vec;              // residual rows are whole, aligned 8-byte words
   int res_q, res_r;         // ceil(s / 16) = res_q n_chunks + res_r
@@ -415,18 +418,22 @@ struct XParams {
   int n_problems, M, n_stages, row_slot;
   int tma;                  // every problem's codes come by TMA (rows of whole 16-byte vectors)
   int total_units;
+  uint32_t shift[8];        // 2^(14 - 2i)
   int* status;              // device status word (the first layout's)
   int cta_u0[kMaxGrid + 1];
 };
 // Words of a layout's partial rows: one CTA per SM with up to 16 words per consumer thread.
 constexpr size_t kXPartWordsPerSm = 16 * 256;
-inline size_t x_smem_bytes(int mt, int row_slot, int n_stages) {
-  return (size_t)n_stages * x_stage_layout(mt, row_slot).total + kMaxProblems * sizeof(XProblem) +
-         2 * (size_t)n_stages * sizeof(unsigned long long) + 256;
+static_assert(kXPartWordsPerSm <= kMbPartFloatsPerCta, "2-bit layouts keep one buffer for both low-batch kernels");
+inline size_t x_smem_bytes(int mode, int mt, int row_slot, int n_stages) {
+  return (size_t)n_stages * x_stage_layout(mode, mt, row_slot).total + kMaxProblems * sizeof(XProblem) +
+         2 * (size_t)n_stages * sizeof(unsigned long long) + 256 + 2048 + (mode <= 1 ? 0 : 1024);
 }
 
 cudaError_t b3mma_configure(size_t smem_optin);
 cudaError_t launch_b3mma(const TensorMaps& maps, const XParams& p, int grid, size_t smem, cudaStream_t st);
+cudaError_t mma2_configure(size_t smem_optin);
+cudaError_t launch_mma2(const TensorMaps& maps, const XParams& p, bool grp, int grid, size_t smem, cudaStream_t st);
 
 // ---------------------------------------------------------------- generic kernel (any M)
 struct GenericParams {
@@ -604,6 +611,7 @@ struct qtea_layout {
   int sm_count;
   size_t smem_optin;
   size_t smem_per_sm;
+  size_t x_smem_optin;   // dynamic shared memory the tensor-core kernel may use
   bool paper_staged_ok;  // the paper-storage kernel with staged activations is configured
   // batch-1 kernel resources
   bool m1_ok;
@@ -617,6 +625,7 @@ struct qtea_layout {
   CUtensorMap tmap8;     // the codes in boxes of 8 rows x 128 bytes (row-resident kernel)
   size_t rows_smem_optin;  // dynamic shared memory the row-resident kernel may use
   // low-batch kernel resources
+  bool mma2_ok;          // the tensor-core kernel with staged B operands takes it (its residual included)
   bool mb_ok;
   size_t mb_smem_optin;
   size_t prep_smem_optin;  // dynamic shared memory the prep kernel may use
@@ -626,7 +635,7 @@ struct qtea_layout {
                          // of every 256-row tile [n_tiles][kMbResFloatsPerTile]
   float* mb_part;        // [sm_count][kMbPartFloatsPerCta] partial rows of split tiles
   unsigned* mb_counters; // [n_tiles of 256 rows][kMbConsumerWarps]
-  // tensor-core base-3 kernel resources (base-3 layouts whose residual it takes)
+  // tensor-core kernel resources (base-3 layouts whose residual it takes; 2-bit layouts use mb_part)
   bool x_ok;
   bool x_tma;            // tmap describes the codes in boxes of 256 rows x kXBoxBytes
   uint32_t* x_part;      // [sm_count][kXPartWordsPerSm]
