@@ -9,6 +9,7 @@ no GPU is present, the calls raise.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 from typing import Optional
 
@@ -112,9 +113,10 @@ def status_string(status: int) -> str:
 
 
 def _stream(stream) -> Optional[int]:
-    import torch
     if stream is None:
-        stream = torch.cuda.current_stream()
+        import torch
+        # the current stream's handle without a Stream object around it (2 us a call)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -133,6 +135,7 @@ def _ptr(t, dtypes, name, shape=None):
     return t.data_ptr()
 
 
+@functools.lru_cache(maxsize=None)
 def _f16_types():
     import torch
     return (torch.float16, torch.int16) + ((torch.uint16,) if hasattr(torch, "uint16") else ())
@@ -209,25 +212,34 @@ def qtea_pack_layout(codes, n_salient: int = 0, group_size: Optional[int] = None
 
 
 def _problem_args(x, layout, row_scale, col_scale, salient_idx, residual_vals, residual_idx, y):
+    # A call of a small layer costs more here than on the GPU: every argument is checked by one expression
+    # that reads each property once, and the checks with messages (_ptr) run for an argument that fails it.
     import torch
-    f16 = _f16_types()
+    T, f16 = torch.Tensor, _f16_types()
     if x.dim() != 2:
         raise ValueError("x must be [M][K]")
     M = x.shape[0]
-    N, K, s = layout.N, layout.K, layout.n_salient
+    N, K, s, options = layout.N, layout.K, layout.n_salient, layout.options
+
+    def ptr(t, dtypes, name, shape):
+        if isinstance(t, T) and t.is_cuda and t.dtype in dtypes and t.is_contiguous() and t.shape == shape:
+            return t.data_ptr()
+        return _ptr(t, dtypes, name, shape)
+
     if y is None:
         y = torch.empty((M, N), dtype=torch.float32, device=x.device)
+    if row_scale is not None and not (isinstance(row_scale, T) and row_scale.dim() == 1):
+        row_scale = row_scale.reshape(-1)
+    u8 = (torch.uint8,)
     args = [
-        _ptr(x, f16, "x", (M, K)),
+        ptr(x, f16, "x", (M, K)),
         layout.handle,
-        _ptr(row_scale.reshape(-1) if row_scale is not None else None, f16, "row_scale",
-             (N * layout.G * (2 if layout.options & QTEA_OPT_BIAS else 1),)),
-        _ptr(col_scale, f16, "col_scale", (K,)),
-        _ptr(salient_idx, (torch.int32,), "salient_idx", (s,)) if s else None,
-        _ptr(residual_vals, (torch.uint8,) if layout.options & QTEA_OPT_RESIDUAL_FP8 else f16, "residual_vals",
-             (N // 4, s)) if s else None,
-        _ptr(residual_idx, (torch.uint8,), "residual_idx", (N // 4, (s + 3) // 4)) if s else None,
-        _ptr(y, (torch.float32,), "y", (M, N)),
+        ptr(row_scale, f16, "row_scale", (N * layout.G * (2 if options & QTEA_OPT_BIAS else 1),)),
+        ptr(col_scale, f16, "col_scale", (K,)),
+        ptr(salient_idx, (torch.int32,), "salient_idx", (s,)) if s else None,
+        ptr(residual_vals, u8 if options & QTEA_OPT_RESIDUAL_FP8 else f16, "residual_vals", (N // 4, s)) if s else None,
+        ptr(residual_idx, u8, "residual_idx", (N // 4, (s + 3) // 4)) if s else None,
+        ptr(y, (torch.float32,), "y", (M, N)),
     ]
     return args, y, M
 
