@@ -776,14 +776,15 @@ __device__ __forceinline__ void x_decode2(const uint8_t* codes, const uint8_t* b
         const float* d = &acc[r >> 1][j][2 * (r & 1)];
         if constexpr (SPLIT) {
           float& t = GRP ? part[r >> 1][j][r & 1] : run[r >> 1][j][r & 1];
-          t = fmaf(a1, (d[0] + d[1]) * fold[4 * j + q], t);
-          if (GRP && bias) t = fmaf(be, sx[16 * blk + 4 * j + q], t);
+          if (GRP) t += fmaf(a1, (d[0] + d[1]) * fold[4 * j + q], bias ? be * sx[16 * blk + 4 * j + q] : 0.f);
+          else t = fmaf(a1, (d[0] + d[1]) * fold[4 * j + q], t);
         } else {
 #pragma unroll
           for (int z = 0; z < 2; ++z) {
-            float& t = run[r >> 1][j][2 * (r & 1) + z];
-            t = fmaf(a1, d[z], t);
-            if (GRP && bias && (w & 1)) t = fmaf(be, sx[16 * blk + 8 * j + 2 * q + z], t);
+            float &t = run[r >> 1][j][2 * (r & 1) + z], &half = part[r >> 1][j][2 * (r & 1) + z];
+            if (!GRP) t = fmaf(a1, d[z], t);
+            else if ((w & 1) == 0) half = d[z];  // joined below: one addition to the tile's sum per group
+            else t += fmaf(a1, half + d[z], bias ? be * sx[16 * blk + 8 * j + 2 * q + z] : 0.f);
           }
         }
       }
