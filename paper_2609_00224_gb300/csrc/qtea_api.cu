@@ -321,7 +321,8 @@ int run_mma(const qtea_gemv_problem* qs, const int* idx, int n, bool base3, int 
     P.n_stages = S;
     int grid = l0->sm_count;
     if (units < grid) grid = (int)units;
-    for (int b = 0; b <= grid; ++b) P.cta_u0[b] = (int)unit_begin_of(b, units, grid);
+    P.unit_q = (int)(units / grid);
+    P.unit_r = (int)(units % grid);
     const size_t smem = x_smem_bytes(mode, mt, P.row_slot, S);
     if ((base3 ? launch_b3mma(maps, P, grid, smem, st) : launch_mma2(maps, P, grp, grid, smem, st)) != cudaSuccess)
       return QTEA_ERR_CUDA;
@@ -698,7 +699,6 @@ bool group_plan(M1Group& g, int sm_count, size_t smem_optin) {
   if (g.gp.total_units >= (1ll << 30)) return false;
   g.grid = (int)(g.gp.total_units < sm_count ? g.gp.total_units : sm_count);
   if (g.grid > kMaxGrid) g.grid = kMaxGrid;
-  for (int b = 0; b <= g.grid; ++b) g.gp.cta_u0[b] = (int)unit_begin_of(b, g.gp.total_units, g.grid);
   for (int stages = kMaxStages; stages >= kMinStages; --stages) {
     if (m1_smem_bytes(stages) <= smem_optin) {
       g.gp.n_stages = stages;
@@ -710,6 +710,7 @@ bool group_plan(M1Group& g, int sm_count, size_t smem_optin) {
 }
 
 int group_launch(M1Group& g, cudaStream_t st) {
+  for (int b = 0; b <= g.grid; ++b) g.gp.cta_u0[b] = (int)unit_begin_of(b, g.gp.total_units, g.grid);
   return launch_m1(g.maps, g.gp, g.grid, g.smem, st) == cudaSuccess ? QTEA_OK : QTEA_ERR_CUDA;
 }
 

@@ -107,6 +107,11 @@ struct GroupParams {
 __host__ __device__ inline long long unit_begin_of(int b, long long total, int grid) {
   return (long long)b * total / grid;
 }
+// The same from total = unit_q grid + unit_r (below 2^31; b unit_r < 2^20), for a kernel that takes no table of
+// them: one among its parameters, 4 KB, cost a launch over 152 CTAs 1.2 us on the host.
+__host__ __device__ inline int cta_unit_begin(unsigned b, int unit_q, int unit_r, unsigned grid) {
+  return (int)(b * (unsigned)unit_q + b * (unsigned)unit_r / grid);
+}
 
 // Dynamic shared memory of the batch-1 kernel with S code stages: codes, auxiliary slots, the
 // helpers' one-hot tables, the problem table, the barriers (code stages: full, empty; auxiliary slots: planes written, residual
@@ -420,7 +425,7 @@ struct XParams {
   int total_units;
   uint32_t shift[8];        // 2^(14 - 2i)
   int* status;              // device status word (the first layout's)
-  int cta_u0[kMaxGrid + 1];
+  int unit_q, unit_r;       // total_units = unit_q grid + unit_r (cta_unit_begin)
 };
 // Words of a layout's partial rows: one CTA per SM with up to 16 words per consumer thread.
 constexpr size_t kXPartWordsPerSm = 16 * 256;

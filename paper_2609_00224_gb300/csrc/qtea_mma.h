@@ -100,7 +100,7 @@ __device__ __forceinline__ void x_part_store(uint32_t* p, uint32_t w) {
   asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(w) : "memory");
 }
 
-// CTA whose range contains unit u (the inverse of the balanced split cta_u0[b] = b * total / grid).
+// CTA whose range contains unit u (the inverse of unit_begin_of).
 __device__ __forceinline__ int x_unit_owner(long long u, long long total, int grid) {
   return (int)(((u + 1) * grid - 1) / total);
 }
@@ -714,7 +714,7 @@ __device__ __forceinline__ void x_step2(const uint8_t* bt, const uint8_t* vt, in
   if (!SPLIT) vp = *reinterpret_cast<const uint2*>(vt + ((4 * w + T) * 4 + q) * 8);
 #pragma unroll
   for (int k = 0; k < BLK; ++k) {
-    uint32_t a0 = x_a2<2 * T, false>(c[2 * k], P), a1 = x_a2<2 * T, false>(c[2 * k + 1], P);
+    uint32_t a0 = x_a2<2 * T, SPLIT>(c[2 * k], P), a1 = x_a2<2 * T, SPLIT>(c[2 * k + 1], P);
     uint32_t a2 = x_a2<2 * T + 1, SPLIT>(c[2 * k], P), a3 = x_a2<2 * T + 1, SPLIT>(c[2 * k + 1], P);
     if (!SPLIT) {
       a0 = x_hmul2(a0, vp.x);
@@ -813,7 +813,8 @@ __global__ void __launch_bounds__(kXThreads, 1)
   extern __shared__ __align__(128) uint8_t smem_raw[];
   uint8_t* smem = smem_raw + (BASE3 ? 0u : (1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int u0 = P.cta_u0[blockIdx.x], u1 = P.cta_u0[blockIdx.x + 1], n_units = u1 - u0;
+  const int u0 = cta_unit_begin(blockIdx.x, P.unit_q, P.unit_r, gridDim.x);
+  const int u1 = cta_unit_begin(blockIdx.x + 1, P.unit_q, P.unit_r, gridDim.x), n_units = u1 - u0;
   const int S = P.n_stages, row_slot = P.row_slot, NP = P.n_problems, M = P.M;
   const XStage lay = x_stage_layout(MODE, MT, row_slot);
   XProblem* tab = reinterpret_cast<XProblem*>(smem + (size_t)S * lay.total);
