@@ -748,15 +748,15 @@ def qtea_arm(args):
     if not args.no_paper:
         paper = {"workload": "llama3_8b_layer_paper_storage", "M": 1,
                  "base3_fp8": dict(paper_leg(qt.QTEA_FMT_BASE3, True),
-                                   kernel="qtea_gemv_lut_kernel<grouped> (the paper's table decode, alpha and "
-                                          "beta per 128 columns staged per tile)"),
+                                   kernel="qtea_gemv_mma_kernel (base-3 digits as fp16 pairs on the tensor cores, "
+                                          "alpha and beta per 128 columns)"),
                  "2bit_fp16_residual": dict(paper_leg(qt.QTEA_FMT_2BIT, False),
                                             kernel="qtea_gemv_m1_kernel, grouped variant (alpha and beta "
                                                    "applied per 128-column group in the decode)")}
 
-    # ---- the paper's decode against the fixed-point one: the Llama3-8B layer in base-3 codes (one
-    #      alpha per row, fp16 residual values), the same resident layouts decoded by the sign-symmetric
-    #      lookup table (Sec. 3.5, Appendix A) and by the fixed-point dot-product kernel
+    # ---- two decodes of base-3 codes: the Llama3-8B layer in base-3 codes (one alpha per row, fp16 residual
+    #      values), the same resident layouts decoded on the tensor cores (the default; the table lookup of
+    #      Sec. 3.5 keeps salient sets too dense for it) and by the fixed-point dot-product kernel
     def lut_leg():
         n_res, nsteps = 4, 16
         shapes = synth.workload_shapes(LAYER_WORKLOAD)
@@ -778,7 +778,7 @@ def qtea_arm(args):
         pbytes = sum(algorithmic_bytes(N, K, synth.salient_count(K)) - N * (-(-K // 64) * 64) // 4
                      + N * (-(-K // 128)) * 26 for _, N, K in shapes)
         out = {}
-        for name, opt in (("lut", 0), ("fixed_point_dp4a", qt.QTEA_OPT_FIXED_POINT)):
+        for name, opt in (("tensor_core", 0), ("fixed_point_dp4a", qt.QTEA_OPT_FIXED_POINT)):
             for L in players:
                 for g in L:
                     g["layout"].set_options(opt)
@@ -795,7 +795,7 @@ def qtea_arm(args):
                 raise RuntimeError(f"device status {status} in the {name} steps")
             out[name] = {"us_per_step": round(tp, 2), "GBps": round(pbytes / (tp * 1e-6) / 1e9, 1),
                          "frac_of_measured_hbm": round(pbytes / (tp * 1e-6) / 1e9 / peak, 3)}
-        out["lut"]["kernel"] = "qtea_gemv_lut_kernel (half-LUT of 122 fp32 entries per code byte)"
+        out["tensor_core"]["kernel"] = "qtea_gemv_mma_kernel (base-3 digits as fp16 pairs, mma.sync)"
         out["fixed_point_dp4a"]["kernel"] = "qtea_gemv_paper_b3_kernel (22/23-bit planes, dp4a)"
         out["bytes_per_step"] = pbytes
         out["layers_resident"] = n_res
