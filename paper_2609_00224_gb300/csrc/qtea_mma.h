@@ -28,7 +28,8 @@
 // extraction, most of them on the logic pipe (64 lanes per clock per SM); that alone would run at 59
 // weights per clock per SM, the MMAs of one n8 tile alone (new A registers every time: 10.9 cycles each per
 // sub-partition) at 94, both together at 50, whether with 8 or 16 decoding warps. 2-bit codes: 67 and together 45
-// (M <= 4). M > 4 adds MMAs, and at M = 16 the consumers decode a unit in 4700 cycles.
+// (M <= 4). M > 4 adds MMAs, and at M = 16 the consumers decode a unit in 4700 cycles, half of
+// them MMAs (sixteen consumer warps of one block, B left as it is, shifts on the multiply pipe: the same).
 // Work split: the units of every problem of a group form one sequence split evenly over one persistent
 // CTA per SM; a tile whose units span several CTAs is finished by the CTA holding its first unit, which
 // reaches it last and adds the others' partial rows in CTA order (self-validating words, as in the
@@ -41,10 +42,12 @@
 // The helpers come first in the CTA and their global loads go out a unit ahead: one set of four, or loads
 // where they are used, made the consumers wait 1000 to 4000 cycles per unit; a third set took registers from
 // the decoding (34.1 us where two give 32.6).
-// Measured, Llama3-8B layer in the paper's storage, seven GEMVs in one call: M = 1 82.3 -> 30.5 us (table
-// lookup before), M = 4 271 -> 34.2 us (fixed-point dp4a before), M = 16 6430 -> 70 us (the general kernel).
-// Qwen3-14B layer, 2-bit codes: M = 4 40.8 -> 32.6 us, M = 16 55.6 -> 54.3 us (both from the low-batch kernel of
-// qtea_gemv_mb.cu, whose pass before the kernel and grid barrier this one does without).
+// Measured, Llama3-8B layer in the paper's storage, seven GEMVs in one call: M = 1 82.4 -> 30.4 us (table
+// lookup before), M = 4 271 -> 34.3 us (fixed-point dp4a before), M = 16 6430 -> 71 us (the general kernel).
+// Qwen3-14B layer, 2-bit codes: M = 4 41.0 -> 32.3 us, M = 16 55.4 -> 53.2 us. Before, the kernel of
+// qtea_gemv_mb.cu, whose pass before the kernel and barrier across the grid this one does without: the barrier's
+// target was part of the launch, so that replays of a captured graph did not wait (34.5 and 49.5 us, and
+// other results than the direct call wherever the activations had changed).
 #pragma once
 
 #include <cuda_fp16.h>
@@ -496,9 +499,11 @@ __device__ __forceinline__ void x_decode_diag(const uint8_t* codes, int row_slot
                                               float (&sum)[BLK][2]) {
   constexpr int R = 2 * BLK;  // the thread's rows: 8 apart
   const int stride = 8 * row_slot;
-  float acc[BLK][4];
+  float acc[2][BLK][4];  // the steps alternate between two sets
 #pragma unroll
-  for (int k = 0; k < BLK; ++k) acc[k][0] = acc[k][1] = acc[k][2] = acc[k][3] = 0.f;
+  for (int k = 0; k < 2 * BLK; ++k)
+#pragma unroll
+    for (int z = 0; z < 4; ++z) acc[k & 1][k >> 1][z] = 0.f;
   uint32_t w[R];
 #pragma unroll
   for (int r = 0; r < R; ++r) w[r] = *reinterpret_cast<const uint32_t*>(codes + r * stride);
@@ -519,7 +524,7 @@ __device__ __forceinline__ void x_decode_diag(const uint8_t* codes, int row_slot
       const uint2 b = *reinterpret_cast<const uint2*>(bt + (5 * u + l) * 256 + (lane ^ (4 * (l & 3))) * 8);
 #pragma unroll
       for (int k = 0; k < BLK; ++k)
-        x_mma(acc[k], e[2 * k].digit(), e[2 * k + 1].digit(), o[2 * k].digit(), o[2 * k + 1].digit(), b);
+        x_mma(acc[(u + l) & 1][k], e[2 * k].digit(), e[2 * k + 1].digit(), o[2 * k].digit(), o[2 * k + 1].digit(), b);
       if (l < 4) {
 #pragma unroll
         for (int r = 0; r < R; ++r) {
@@ -544,12 +549,12 @@ __device__ __forceinline__ void x_decode_diag(const uint8_t* codes, int row_slot
       e[r].next();
     }
 #pragma unroll
-    for (int k = 0; k < BLK; ++k) x_mma(acc[k], a0[2 * k], a0[2 * k + 1], a1[2 * k], a1[2 * k + 1], b);
+    for (int k = 0; k < BLK; ++k) x_mma(acc[(l >> 1) & 1][k], a0[2 * k], a0[2 * k + 1], a1[2 * k], a1[2 * k + 1], b);
   }
 #pragma unroll
   for (int k = 0; k < BLK; ++k) {
-    sum[k][0] = acc[k][0] + acc[k][1];
-    sum[k][1] = acc[k][2] + acc[k][3];
+    sum[k][0] = (acc[0][k][0] + acc[1][k][0]) + (acc[0][k][1] + acc[1][k][1]);
+    sum[k][1] = (acc[0][k][2] + acc[1][k][2]) + (acc[0][k][3] + acc[1][k][3]);
   }
 }
 
@@ -735,7 +740,7 @@ constexpr int kXFoldV = 2;
 // at segment w ^ (row % 8)). SPLIT: B holds (hi, lo) of v*x 2^E / 2, folded with 2^-E; else A = 2T * v, one exact
 // fp16 multiply by the pairs in vt, and B holds x. GRP: the accumulators are folded per 128-column group with
 // the rows' alpha and beta of the group (staged at sc), else per unit with the row's alpha (al); with v in A,
-// whose products have 22 bits, after every half group (GRP) or two words. run: [block]
+// whose products have 22 bits, two or four times a unit. run: [block]
 // [tile][value]: SPLIT rows g, g + 8 of batch row 4 tile + q; else (row, batch row 8 tile + 2q + 0 / 1).
 template <int MT, int BLK, bool SPLIT, bool GRP>
 __device__ __forceinline__ void x_decode2(const uint8_t* codes, const uint8_t* bt, const uint8_t* vt, const uint8_t* sc,
@@ -743,23 +748,28 @@ __device__ __forceinline__ void x_decode2(const uint8_t* codes, const uint8_t* b
                                           int g, int q, int lane, const XParams& P,
                                           float (&run)[BLK][MT][SPLIT ? 2 : 4]) {
   constexpr int R = 2 * BLK, NV = SPLIT ? 2 : 4;
-  constexpr int kFold = SPLIT ? (GRP ? 2 : 8) : (GRP ? 1 : 2);  // words (four steps each) per fold
-  float acc[BLK][MT][4], part[BLK][MT][NV];
+  // The steps alternate between two sets of accumulators: half the chain, and MMAs that do not wait for one
+  // another (14b layer, M = 16: 54.3 -> 53.2 us); with one tile and v in A one set folded twice as often is
+  // faster (M = 8: 39.1 us; 40.2 with two).
+  constexpr bool kTwo = SPLIT || GRP || MT > 1;
+  constexpr int kFold = GRP ? 2 : (SPLIT ? 8 : (kTwo ? 4 : 2));  // words (four steps each) per fold
+  float acc[2][BLK][MT][4], part[BLK][MT][NV];
 #pragma unroll
   for (int k = 0; k < BLK; ++k)
 #pragma unroll
     for (int j = 0; j < MT; ++j)
 #pragma unroll
       for (int z = 0; z < NV; ++z) part[k][j][z] = 0.f;
-#pragma unroll (SPLIT || !GRP ? 8 : 2)  // two: the staged scales leave too few registers for eight
+#pragma unroll (SPLIT || (MT == 1 && !GRP) ? 8 : (GRP ? 2 : 4))  // registers
   for (int w = 0; w < 8; ++w) {
     uint32_t c[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) c[r] = *reinterpret_cast<const uint32_t*>(codes + r * 1024 + ((w ^ g) << 4));
-    x_step2<MT, BLK, SPLIT, 0>(bt, vt, w, q, lane, c, w % kFold == 0, P, acc);
-    x_step2<MT, BLK, SPLIT, 1>(bt, vt, w, q, lane, c, false, P, acc);
-    x_step2<MT, BLK, SPLIT, 2>(bt, vt, w, q, lane, c, false, P, acc);
-    x_step2<MT, BLK, SPLIT, 3>(bt, vt, w, q, lane, c, false, P, acc);
+    const bool first = w % kFold == 0;
+    x_step2<MT, BLK, SPLIT, 0>(bt, vt, w, q, lane, c, first, P, acc[0]);
+    x_step2<MT, BLK, SPLIT, 1>(bt, vt, w, q, lane, c, first && kTwo, P, acc[kTwo ? 1 : 0]);
+    x_step2<MT, BLK, SPLIT, 2>(bt, vt, w, q, lane, c, false, P, acc[0]);
+    x_step2<MT, BLK, SPLIT, 3>(bt, vt, w, q, lane, c, false, P, acc[kTwo ? 1 : 0]);
     if (w % kFold != kFold - 1) continue;
     const int blk = w >> 1;
 #pragma unroll
@@ -773,18 +783,18 @@ __device__ __forceinline__ void x_decode2(const uint8_t* codes, const uint8_t* b
       if (!SPLIT) a1 *= 0.5f;
 #pragma unroll
       for (int j = 0; j < MT; ++j) {
-        const float* d = &acc[r >> 1][j][2 * (r & 1)];
+        const float *d = &acc[0][r >> 1][j][2 * (r & 1)], *e = &acc[1][r >> 1][j][2 * (r & 1)];
         if constexpr (SPLIT) {
           float& t = GRP ? part[r >> 1][j][r & 1] : run[r >> 1][j][r & 1];
-          if (GRP) t += fmaf(a1, (d[0] + d[1]) * fold[4 * j + q], bias ? be * sx[16 * blk + 4 * j + q] : 0.f);
-          else t = fmaf(a1, (d[0] + d[1]) * fold[4 * j + q], t);
+          const float sum = ((d[0] + e[0]) + (d[1] + e[1])) * fold[4 * j + q];
+          if (GRP) t += fmaf(a1, sum, bias ? be * sx[16 * blk + 4 * j + q] : 0.f);
+          else t = fmaf(a1, sum, t);
         } else {
 #pragma unroll
           for (int z = 0; z < 2; ++z) {
-            float &t = run[r >> 1][j][2 * (r & 1) + z], &half = part[r >> 1][j][2 * (r & 1) + z];
-            if (!GRP) t = fmaf(a1, d[z], t);
-            else if ((w & 1) == 0) half = d[z];  // joined below: one addition to the tile's sum per group
-            else t += fmaf(a1, half + d[z], bias ? be * sx[16 * blk + 8 * j + 2 * q + z] : 0.f);
+            float& t = run[r >> 1][j][2 * (r & 1) + z];
+            if (GRP) t += fmaf(a1, d[z] + e[z], bias ? be * sx[16 * blk + 8 * j + 2 * q + z] : 0.f);
+            else t = fmaf(a1, kTwo ? d[z] + e[z] : d[z], t);
           }
         }
       }
