@@ -555,14 +555,15 @@ bool mb_group_add(MbGroup& g, const qtea_gemv_problem& q) {
 }
 
 // Grid, ring depth and shared memory of the group; false if the ring does not fit.
-bool mb_group_plan(MbGroup& g, int sm_count, size_t smem_optin) {
+bool mb_group_plan(MbGroup& g, int sm_count, size_t smem_optin, bool captured) {
   if (g.gp.n_problems == 0) return false;
   if (g.gp.total_units >= (1ll << 30)) return false;
   g.grid = (int)(g.gp.total_units < sm_count ? g.gp.total_units : sm_count);
   if (g.grid > kMaxGrid) g.grid = kMaxGrid;
   for (int b = 0; b <= g.grid; ++b) g.gp.cta_u0[b] = (int)unit_begin_of(b, g.gp.total_units, g.grid);
-  // no residual left to the prep kernel: its other work moves into the main kernel (one launch)
-  g.gp.fused = 1;
+  // no residual left to the prep kernel: its other work moves into the main kernel (one launch), but not in a
+  // graph: the grid barrier's target is part of the launch, and a replay would find the counter past it
+  g.gp.fused = captured ? 0 : 1;
   for (int k = 0; k < g.gp.n_problems; ++k)
     if (g.gp.prob[k].res_mode == kMbResPrep) g.gp.fused = 0;
   if (g.gp.fused) {
@@ -606,6 +607,8 @@ bool mb_capable(const qtea_layout* l, int M) {
 // Low-batch dispatch: as many consecutive problems per launch as fit (one kernel variant per
 // launch); a problem the kernel cannot take goes to the paper-storage or the generic kernel.
 int run_mb(const qtea_gemv_problem* qs, const int* idx, int n, int M, cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  const bool captured = cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone;
   int i = 0;
   while (i < n) {
     const qtea_layout* l0 = qs[idx[i]].packed_ternary;
@@ -617,7 +620,7 @@ int run_mb(const qtea_gemv_problem* qs, const int* idx, int n, int M, cudaStream
       if (li->sm_count != l0->sm_count) break;  // partial-row slots are sized by the SM count
       MbGroup trial = g;
       if (!mb_group_add(trial, qs[idx[i + taken]])) break;
-      if (!mb_group_plan(trial, l0->sm_count, l0->mb_smem_optin)) break;
+      if (!mb_group_plan(trial, l0->sm_count, l0->mb_smem_optin, captured)) break;
       g = trial;
       ++taken;
     }

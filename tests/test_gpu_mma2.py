@@ -116,3 +116,24 @@ def test_extreme_scales(qt, M, value, which):
     q["row_scale" if which == "alpha" else "col_scale"].copy_(
         dev(np.ascontiguousarray(getattr(p, which)).reshape(-1).view(np.int16), torch.float16))
     check(p, qt.qtea_gemv(**q), False)
+
+
+@pytest.mark.parametrize("M", [3, 12])
+def test_dense_salient_set_graph_replay(qt, M):
+    """The older low-batch kernel, captured in a graph and replayed on other activations: as the direct call."""
+    items = [problem(qt, N, 2048, M, 512, g, False, False, seed=90 + i) for i, (N, g) in enumerate([(4096, 0), (2048, 128)])]
+    probs = [dict(q, y=torch.empty((M, p.N), dtype=torch.float32, device="cuda")) for p, q in items]
+    st, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    st.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.graph(graph, stream=st):
+        qt.qtea_gemv_grouped(probs)
+    for _ in range(5):
+        for q in probs:
+            q["x"].copy_(torch.randn(q["x"].shape, device="cuda").half())
+        graph.replay()
+        torch.cuda.synchronize()
+        y = [q["y"].clone() for q in probs]
+        qt.qtea_gemv_grouped(probs)
+        torch.cuda.synchronize()
+        for a, q in zip(y, probs):
+            assert float((a - q["y"]).norm() / q["y"].norm()) < 1e-6
