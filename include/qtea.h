@@ -100,13 +100,13 @@ typedef enum qtea_option {
  * columns, and fit one such launch: at most 32 rows per CTA with one or two CTAs per SM, one when
  * some problem has K > 4096 or more than 256 salient columns;
  * a latency-bound form for small calls), else the persistent stream-K launch; the tensor-core
- * low-batch kernel takes those at M >= 2 and 2-bit layouts with FP8 residual values (groups of 128
- * columns, or beta absent) at any M; base-3 layouts run on the tensor-core base-3 kernel at any M, but
- * for the following: at M = 1 with QTEA_OPT_FIXED_POINT on a kernel that stages v*x once per CTA in
- * fixed point; layouts with so many salient columns that a 512-column chunk's share exceeds 32 of them
- * on the paper's table-lookup decode (M = 1; Sec. 3.5, Appendix A), that fixed-point kernel (M <= 4) or
- * a general kernel; the rest run on general kernels. The problems of a grouped call that the same
- * kernel serves share launches.
+ * kernel takes 2-bit layouts at M >= 2, those with FP8 residual values at any M, and base-3 layouts at
+ * any M, but for the following. Layouts with so many salient columns that a 512-column chunk's share
+ * exceeds 32 of them: 2-bit ones on an older low-batch kernel or a general kernel, base-3 ones on the
+ * paper's table-lookup decode (M = 1; Sec. 3.5, Appendix A), a kernel that stages v*x once per CTA in
+ * fixed point (M <= 4; at M = 1 for any base-3 layout with QTEA_OPT_FIXED_POINT) or a general kernel.
+ * The rest run on general kernels. The problems of a grouped call that the same kernel serves share
+ * launches.
  *
  * The call validates every code on the device and synchronizes `stream` once to read the
  * result; invalid codes give QTEA_ERR_BAD_CODES and no layout. It allocates the packed
@@ -146,12 +146,11 @@ int qtea_pack_layout(const int8_t* ternary_codes, int N, int K, int group_size, 
  * Numerics: at M = 1 (the library's own storage) the ternary sum is accumulated exactly in
  * integers over 512-column blocks, with v*x represented in 16-bit or 24-bit fixed point relative
  * to the block's largest |v*x| after its massive values are taken out and added exactly in fp32
- * (qtea_set_activation_precision); block sums, alpha and the residual are combined in fp32. At 2 <= M <= 16, and for 2-bit layouts in the paper's
- * storage at any M, the tensor cores take 2T*v and x in fp16 (both exact, which needs |v| < 32768)
- * with exact fp32 products and fp32 sums; alpha, beta and the residual are applied in fp32.
- * Base-3 layouts on the tensor-core kernel: 2T and v*x (as an fp16 pair whose sum is exact to 22 bits
- * of the largest of its 512 columns) are exact, products are summed on the tensor cores over at most
- * 512 columns, the rest in fp32 (infinities and NaN in v*x make the batch row NaN). On the fixed-point
+ * (qtea_set_activation_precision); block sums, alpha and the residual are combined in fp32. On the
+ * tensor-core kernel 2T and v*x (as an fp16 pair whose sum is exact to 22 bits of the largest of its 512
+ * columns) are exact, products are summed on the tensor cores over at most 512 columns, the rest in fp32
+ * (infinities and NaN in v*x make the batch row NaN); 2-bit layouts at M >= 5, and the older low-batch
+ * kernel, take 2T*v and x in fp16 (both exact, which needs |v| < 32768). On the fixed-point
  * kernel (when v*x of the call fits in shared memory): the ternary sum is accumulated exactly in integers over 128-column blocks, with v*x in fixed point relative to the
  * block's largest |v*x| (|X| < 2^23) after up to 3 massive values per block are taken out and
  * added exactly in fp32; block sums, alpha, beta and the residual are combined in fp32. Other
@@ -176,7 +175,7 @@ typedef struct qtea_gemv_problem {
 /*
  * Several independent GEMVs with the same batch M, as if qtea_gemv were called for each in
  * order, but sharing launches: up to 8 consecutive problems that the same kernel variant serves
- * (batch 1; low batch with one alpha per row; low batch with scale groups) run in one persistent
+ * (batch 1; tensor cores with one alpha per row; with scale groups or beta; base-3) run in one persistent
  * launch, which removes per-launch ramp-up and tail time when the problems are small (e.g. the
  * q/k/v/o/gate/up/down GEMVs of one decoder layer).
  * Every problem is validated before anything is launched; a failing check returns its status
@@ -192,7 +191,7 @@ typedef enum qtea_kernel {
   QTEA_KERNEL_ROWS = 1,         /* batch-1, row-resident launch */
   QTEA_KERNEL_STREAM_K = 2,     /* batch-1, persistent stream-K launch */
   QTEA_KERNEL_LUT = 3,          /* the paper's table-lookup decode (base-3 codes, M = 1) */
-  QTEA_KERNEL_LOW_BATCH = 4,    /* tensor-core low-batch kernel (2-bit codes) */
+  QTEA_KERNEL_LOW_BATCH = 4,    /* tensor-core kernels for 2-bit codes */
   QTEA_KERNEL_BASE3_FIXED = 5,  /* base-3 codes, v*x staged once per CTA in fixed point */
   QTEA_KERNEL_PAPER = 6,        /* general kernel for the paper's storage */
   QTEA_KERNEL_GENERIC = 7,      /* general kernel */
