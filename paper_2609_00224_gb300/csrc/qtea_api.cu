@@ -58,8 +58,9 @@ bool x_shape_ok(const qtea_layout* l, const cudaDeviceProp& prop) {
 }
 
 // Resources of the batch-1 kernel for one layout: its TMA descriptor (512-row x 512-column
-// units, two 256-row boxes each) and the split-tile workspace.
-int plan_m1(qtea_layout* l, const cudaDeviceProp& prop) {
+// units, two 256-row boxes each) and the split-tile workspace. Here and below the workspaces are zeroed on the
+// caller's stream, which the pack call synchronizes: a non-blocking stream does not wait for the default one.
+int plan_m1(qtea_layout* l, const cudaDeviceProp& prop, cudaStream_t st) {
   l->m1_ok = false;
   l->sm_count = prop.multiProcessorCount;
   l->smem_optin = prop.sharedMemPerBlockOptin;
@@ -116,23 +117,23 @@ int plan_m1(qtea_layout* l, const cudaDeviceProp& prop) {
           cudaMalloc(&l->mb_part, (size_t)l->sm_count * kMbPartFloatsPerCta * sizeof(float)) != cudaSuccess ||
           cudaMalloc(&l->mb_counters, ctr) != cudaSuccess)
         return QTEA_ERR_ALLOC;
-      if (cudaMemset(l->mb_counters, 0, ctr) != cudaSuccess) return QTEA_ERR_CUDA;
+      if (cudaMemsetAsync(l->mb_counters, 0, ctr, st) != cudaSuccess) return QTEA_ERR_CUDA;
       // partial rows of split tiles: zero reads as "not written yet"; completed calls leave it zero
-      if (cudaMemset(l->mb_part, 0, (size_t)l->sm_count * kMbPartFloatsPerCta * sizeof(float)) != cudaSuccess)
+      if (cudaMemsetAsync(l->mb_part, 0, (size_t)l->sm_count * kMbPartFloatsPerCta * sizeof(float), st) != cudaSuccess)
         return QTEA_ERR_CUDA;
       if (cudaMalloc(&l->mb_gbar, sizeof(unsigned long long)) != cudaSuccess) return QTEA_ERR_ALLOC;
-      if (cudaMemset(l->mb_gbar, 0, sizeof(unsigned long long)) != cudaSuccess) return QTEA_ERR_CUDA;
+      if (cudaMemsetAsync(l->mb_gbar, 0, sizeof(unsigned long long), st) != cudaSuccess) return QTEA_ERR_CUDA;
       l->mb_gbar_next = 0;
     }
   }
   if (cudaMalloc(&l->workspace, (size_t)l->sm_count * 2 * kTileRows * sizeof(float)) != cudaSuccess)
     return QTEA_ERR_ALLOC;
   // split-tile partial rows: zero reads as "not written yet", and every completed call leaves it zero
-  if (cudaMemset(l->workspace, 0, (size_t)l->sm_count * 2 * kTileRows * sizeof(float)) != cudaSuccess)
+  if (cudaMemsetAsync(l->workspace, 0, (size_t)l->sm_count * 2 * kTileRows * sizeof(float), st) != cudaSuccess)
     return QTEA_ERR_CUDA;
   if (cudaMalloc(&l->counters, (size_t)l->n_tiles * kConsumerWarps * sizeof(unsigned)) != cudaSuccess)
     return QTEA_ERR_ALLOC;
-  if (cudaMemset(l->counters, 0, (size_t)l->n_tiles * kConsumerWarps * sizeof(unsigned)) != cudaSuccess)
+  if (cudaMemsetAsync(l->counters, 0, (size_t)l->n_tiles * kConsumerWarps * sizeof(unsigned), st) != cudaSuccess)
     return QTEA_ERR_CUDA;
   l->m1_ok = true;
   return QTEA_OK;
@@ -140,7 +141,7 @@ int plan_m1(qtea_layout* l, const cudaDeviceProp& prop) {
 
 // Resources of the tensor-core kernel for a base-3 layout: the partial rows of split tiles. Taken when
 // no chunk's share of the salient entries exceeds what a unit stages.
-int plan_b3mma(qtea_layout* l, const cudaDeviceProp& prop) {
+int plan_b3mma(qtea_layout* l, const cudaDeviceProp& prop, cudaStream_t st) {
   l->x_ok = false;
   if (l->N == 0 || l->K == 0) return QTEA_OK;
   if (!x_shape_ok(l, prop)) return QTEA_OK;
@@ -158,13 +159,13 @@ int plan_b3mma(qtea_layout* l, const cudaDeviceProp& prop) {
   }
   const size_t bytes = (size_t)l->sm_count * kXPartWordsPerSm * sizeof(uint32_t);
   if (cudaMalloc(&l->x_part, bytes) != cudaSuccess) return QTEA_ERR_ALLOC;
-  if (cudaMemset(l->x_part, 0, bytes) != cudaSuccess) return QTEA_ERR_CUDA;
+  if (cudaMemsetAsync(l->x_part, 0, bytes, st) != cudaSuccess) return QTEA_ERR_CUDA;
   l->x_ok = true;
   return QTEA_OK;
 }
 
 // Resources of the table-lookup kernel for a base-3 layout: split-tile workspace and counters.
-int plan_lut(qtea_layout* l, const cudaDeviceProp& prop) {
+int plan_lut(qtea_layout* l, const cudaDeviceProp& prop, cudaStream_t st) {
   l->lut_ok = false;
   if (l->N == 0 || l->K == 0) return QTEA_OK;
   if (lut_configure(prop.sharedMemPerBlockOptin) != cudaSuccess) {
@@ -176,7 +177,7 @@ int plan_lut(qtea_layout* l, const cudaDeviceProp& prop) {
   if (cudaMalloc(&l->lut_ws, (size_t)prop.multiProcessorCount * 2 * kLutTileRows * sizeof(float)) != cudaSuccess ||
       cudaMalloc(&l->lut_counters, ctr) != cudaSuccess)
     return QTEA_ERR_ALLOC;
-  if (cudaMemset(l->lut_counters, 0, ctr) != cudaSuccess) return QTEA_ERR_CUDA;
+  if (cudaMemsetAsync(l->lut_counters, 0, ctr, st) != cudaSuccess) return QTEA_ERR_CUDA;
   l->lut_ok = true;
   return QTEA_OK;
 }
@@ -1041,10 +1042,10 @@ int qtea_pack_layout(const int8_t* ternary_codes, int N, int K, int group_size, 
   } else if (cudaMemsetAsync(l->status, 0, 2 * sizeof(int), st) != cudaSuccess) {
     rc = QTEA_ERR_CUDA;
   } else if (format == QTEA_FMT_2BIT) {
-    rc = plan_m1(l, prop);  // the batch-1 and low-batch kernels' resources
+    rc = plan_m1(l, prop, st);  // the batch-1 and low-batch kernels' resources
   } else {
-    rc = plan_b3mma(l, prop);  // the tensor-core base-3 kernel's, else the table-lookup kernel's
-    if (rc == QTEA_OK && !l->x_ok) rc = plan_lut(l, prop);
+    rc = plan_b3mma(l, prop, st);  // the tensor-core base-3 kernel's, else the table-lookup kernel's
+    if (rc == QTEA_OK && !l->x_ok) rc = plan_lut(l, prop, st);
   }
   if (rc == QTEA_OK && cudaStreamSynchronize(st) != cudaSuccess) rc = QTEA_ERR_CUDA;
   if (rc != QTEA_OK) {
