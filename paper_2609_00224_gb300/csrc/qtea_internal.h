@@ -373,6 +373,7 @@ constexpr int kXMaxChunks = 16384;                             // of a layout
 constexpr int kXResSteps = 2;                                  // residual steps (16 entries) a unit may take
 constexpr int kXResBBytes = kXResSteps * 32 * 8;               // their B per tile
 constexpr int kXResStride = 32 * kXResSteps + 8;               // their values per group of four rows
+constexpr int kXOutWords = 16;                                 // words that tell the rows with products left out of B
 constexpr int kXHelpers = 4;                                   // warps of a helper set
 constexpr int kXBlocks = 2;                                    // 16-row blocks of a consumer warp
 constexpr int kXSets = 2;                                      // helper sets
@@ -432,7 +433,7 @@ constexpr size_t kXPartWordsPerSm = 16 * 256;
 static_assert(kXPartWordsPerSm <= kMbPartFloatsPerCta, "2-bit layouts keep one buffer for both low-batch kernels");
 inline size_t x_smem_bytes(int mode, int mt, int row_slot, int n_stages) {
   return (size_t)n_stages * x_stage_layout(mode, mt, row_slot).total + kMaxProblems * sizeof(XProblem) +
-         2 * (size_t)n_stages * sizeof(unsigned long long) + 256 + 2048 + (mode <= 1 ? 0 : 1024);
+         2 * (size_t)n_stages * sizeof(unsigned long long) + 256 + 2048 + 4 * (kXOutWords + 1) + (mode <= 1 ? 0 : 1024);
 }
 
 cudaError_t b3mma_configure(size_t smem_optin);

@@ -14,8 +14,10 @@
 //    c = T + 1 into the fp16 pair 2T = -2, -0 or +2 (sign bit and top exponent bit). 2-bit codes are shifted to
 //    the same two bits.
 //  * B (activations): v*x is exact in fp32; times 2^E (E per chunk and batch row, so that the largest
-//    is below 2^14 after the halving that 2T asks for) it is held as two fp16 columns, hi and lo, whose
-//    sum is exact. Four batch rows make one n8 tile. The sums are folded with 2^-E per chunk. 2-bit codes at
+//    is below 2^15 after the halving that 2T asks for) it is held as two fp16 columns, hi and lo, whose
+//    sum hi + lo / 2^11 is exact down to 2^-28 of the chunk's largest. What it lacks of smaller products, infinities
+//    and NaN are added in fp32 at the end of the tile, to the rows whose code there is not 0. Four batch
+//    rows make one n8 tile. The sums are folded with 2^-E per chunk. 2-bit codes at
 //    M >= 5 have v in A instead (2T * v, one exact fp16 multiply) and x in B, eight batch rows to a tile: half the
 //    MMAs (at M = 16 the decoding loop alone runs at 38 weights per clock per SM, with four split tiles at 27).
 //  * Scales: base-3 at M = 1: column pair q of the tile is non-zero only in the k slots of lane q, so that a
@@ -42,9 +44,11 @@
 // The helpers come first in the CTA and their global loads go out a unit ahead: one set of four, or loads
 // where they are used, made the consumers wait 1000 to 4000 cycles per unit; a third set took registers from
 // the decoding (34.1 us where two give 32.6).
-// Measured, Llama3-8B layer in the paper's storage, seven GEMVs in one call: M = 1 82.4 -> 30.4 us (table
-// lookup before), M = 4 271 -> 34.3 us (fixed-point dp4a before), M = 16 6430 -> 71 us (the general kernel).
-// Qwen3-14B layer, 2-bit codes: M = 4 41.0 -> 32.3 us, M = 16 55.4 -> 53.2 us. Before, the kernel of
+// Measured, Llama3-8B layer in the paper's storage, seven GEMVs in one call: M = 1 82.4 -> 30.8 us (table
+// lookup before), M = 4 271 -> 34.8 us (fixed-point dp4a before), M = 16 6430 -> 71 us (the general kernel).
+// Qwen3-14B layer, 2-bit codes: M = 4 41.0 -> 32.5 us, M = 16 55.4 -> 53.2 us. (With the remainder in lo itself and no
+// search for products below its range, 30.4, 34.3, 71.3 and 32.3 us, and errors up to 2^-39 of a chunk's largest
+// product: 1 to 2 % of a row's sum |x W^| where activations of 5e-7 stand beside one of 6e4 whose code is 0.) Before, the kernel of
 // qtea_gemv_mb.cu, whose pass before the kernel and barrier across the grid this one does without: the barrier's
 // target was part of the launch, so that replays of a captured graph did not wait (34.5 and 49.5 us, and
 // other results than the direct call wherever the activations had changed).
@@ -191,8 +195,10 @@ __device__ __forceinline__ uint32_t x_b_offset(int c) {
   return base + 1280 + half_step + 2 * (w - 4);
 }
 
-// Sixteen columns of x (rows m0, m0 + step, ...) and v per lane: columns 16 lane .. 16 lane + 15 of chunk ch, zero
-// past K and from row M on.
+__device__ __forceinline__ bool x_finite(uint16_t h) { return (h & 0x7C00u) != 0x7C00u; }
+
+// Sixteen columns of x (rows m0, m0 + step, ...) and v per lane: columns 16 lane .. 16 lane + 15 of chunk ch; past K
+// x is zero and v one, and x zero from row M on.
 template <int R>
 struct XRows {
   uint32_t x[R][8], v[8];
@@ -207,7 +213,7 @@ __device__ __forceinline__ void x_load_rows(const XProblem& a, int ch, int m0, i
     const int m = m0 + k * step;
     const uint16_t* src = k < 0 ? a.v + col : a.x + (size_t)m * a.K + col;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) d[i] = 0u;
+    for (int i = 0; i < 8; ++i) d[i] = k < 0 && a.xv_vec ? 0x3C003C00u : 0u;
     if (k < 0 ? !with_v : m >= M) continue;
     if (a.xv_vec) {  // rows of whole 16-byte vectors, 16-byte aligned
 #pragma unroll
@@ -219,44 +225,184 @@ __device__ __forceinline__ void x_load_rows(const XProblem& a, int ch, int m0, i
     } else {
 #pragma unroll
       for (int i = 0; i < 16; ++i)
-        if (col + i < a.K) d[i >> 1] |= (uint32_t)__ldg(src + i) << (16 * (i & 1));
+        d[i >> 1] |= (uint32_t)(col + i < a.K ? __ldg(src + i) : k < 0 ? (uint16_t)0x3C00 : (uint16_t)0) << (16 * (i & 1));
     }
   }
 }
 
+// v*x as an fp16 pair: f = v*x 2^(E - 1) below 2^15 (half of 2^E, since A is 2T), hi = f rounded, lo = the
+// remainder times 2^11, so that the pair is hi + lo / 2^11. f has 22 bits: above 2^-14 the pair is f itself (hi and
+// the remainder's 11 bits are normal, or the remainder is a multiple of 2^-35). What the pair lacks of smaller products
+// (2^-28 of the chunk's largest), and infinities and NaN, the consumers add in fp32 (x_left_out).
+constexpr float kXLo = 0x1p-11f;
+// The product of the two fp16 halves i (0: low), exact in fp32, and a half's addition to an fp32 sum: mixed-precision
+// instructions (PTX ISA 8.6, sm_100 and up), one each where two conversions and the operation would be two or three.
+__device__ __forceinline__ uint16_t x_half(uint32_t w, int i) { return (uint16_t)(w >> (16 * i)); }
+__device__ __forceinline__ float x_fma16(uint16_t a, uint16_t b, float c) {
+  float d;
+  asm("fma.rn.f32.f16 %0, %1, %2, %3;" : "=f"(d) : "h"(a), "h"(b), "f"(c));
+  return d;
+}
+__device__ __forceinline__ float x_add16(uint16_t a, float c) {
+  float d;
+  asm("add.rn.f32.f16 %0, %1, %2;" : "=f"(d) : "h"(a), "f"(c));
+  return d;
+}
+__device__ __forceinline__ float x_max_nan(float a, float b) {  // NaN when either is
+  float d;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+  return d;
+}
+// The pair of two products: hi = RN(p sc), lo = (p sc - hi) 2^11, both from p in one exact step each.
+__device__ __forceinline__ void x_pair(float p0, float p1, float sc, __half2& hi, __half2& lo) {
+  hi = __floats2half2_rn(p0 * sc, p1 * sc);
+  const uint32_t h = *reinterpret_cast<const uint32_t*>(&hi);
+  const float sc2 = sc * 2048.f;
+  lo = __floats2half2_rn(x_fma16(x_half(h, 0), 0xE800u, p0 * sc2), x_fma16(x_half(h, 1), 0xE800u, p1 * sc2));  // -2048
+}
+// 2 |p| in the float's bits, without the sign: 0 for zero, from kXInf on infinities and NaN.
+__device__ __forceinline__ uint32_t x_mag(float p) { return __float_as_uint(p) << 1; }
+constexpr uint32_t kXInf = 0xFF000000u;
+// What the pair lacks of a product, sc = 2^(E - 1): exact, a multiple of fp16's smallest product 2^-48; infinities and
+// NaN whole.
+__device__ __forceinline__ float x_lacking(float p, float sc) {
+  if (x_mag(p) >= kXInf) return p;
+  __half2 hi, lo;
+  x_pair(p, 0.f, sc, hi, lo);
+  return fmaf(-__low2float(lo), kXLo, fmaf(p, sc, -__low2float(hi))) / sc;
+}
+// f(i, product i of the lane's sixteen) of batch row m in chunk ch, read from global memory eight columns at a time: for
+// what runs rarely, in functions of its own. (As part of the kernel's loops that code cost a call of one unit per CTA
+// 0.3 us and the Llama3-8B layer in the paper's storage up to 6, although it never ran.)
+template <typename F>
+__device__ __forceinline__ void x_products(const XProblem& a, int ch, int m, int lane, const F& f) {
+#pragma unroll 1
+  for (int h = 0; h < 2; ++h) {
+    const int col = ch * kXChunkCols + 16 * lane + 8 * h;
+    const uint16_t *x = a.x + (size_t)m * a.K + col, *v = a.v + col;
+    uint4 xw = make_uint4(0u, 0u, 0u, 0u), vw = xw;
+    if (a.xv_vec) {
+      if (col < a.K) {
+        xw = __ldg(reinterpret_cast<const uint4*>(x));
+        vw = __ldg(reinterpret_cast<const uint4*>(v));
+      }
+    } else {
+      uint32_t xs[4] = {0u, 0u, 0u, 0u}, vs[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (col + i < a.K) {
+          xs[i >> 1] |= (uint32_t)__ldg(x + i) << (16 * (i & 1));
+          vs[i >> 1] |= (uint32_t)__ldg(v + i) << (16 * (i & 1));
+        }
+      xw = make_uint4(xs[0], xs[1], xs[2], xs[3]);
+      vw = make_uint4(vs[0], vs[1], vs[2], vs[3]);
+    }
+    const uint32_t xs[4] = {xw.x, xw.y, xw.z, xw.w}, vs[4] = {vw.x, vw.y, vw.z, vw.w};
+#pragma unroll
+    for (int i = 0; i < 8; ++i) f(8 * h + i, x_fma16(x_half(vs[i >> 1], i & 1), x_half(xs[i >> 1], i & 1), 0.f));
+  }
+}
+__device__ __forceinline__ int x_lane() {
+  int lane;
+  asm volatile("mov.u32 %0, %%laneid;" : "=r"(lane));
+  return lane;
+}
+// A row's factors from e, the binade of its largest |v*x| (< 2^(e + 1)).
+__device__ __forceinline__ float x_sc(int e) { return __uint_as_float((uint32_t)(127 + 14 - e) << 23); }    // 2^(E - 1)
+__device__ __forceinline__ float x_fold(int e) { return __uint_as_float((uint32_t)(127 - 15 + e) << 23); }  // 2^-E
+__device__ __forceinline__ int x_binade(float lmax) {  // lmax: the lane's largest; 128 with an infinity or NaN
+  const uint32_t amax = __reduce_max_sync(0xffffffffu, __float_as_uint(lmax));
+  return amax ? (int)(amax >> 23) - 127 : 0;
+}
+// The least |v| of the lane's sixteen columns, in fp16 bits.
+__device__ __forceinline__ uint32_t x_least(const uint32_t (&v)[8]) {
+  uint32_t m = v[0] & 0x7FFF7FFFu;
+#pragma unroll
+  for (int i = 1; i < 8; ++i) m = __vminu2(m, v[i] & 0x7FFF7FFFu);
+  return min(m & 0xFFFFu, m >> 16);
+}
+// The lane's pairs may lack something (then x_search looks): not when the least |v| times fp16's smallest x, 2^-24,
+// or else the row's least x but for zeros, is at least 2^-28 of the binade 2^e. The first spares most chunks the
+// second: 2^e <= 16 with v near 1.
+__device__ __forceinline__ int x_exponent(uint32_t h) { return h >= 0x400u ? (int)(h >> 10) - 15 : -24; }
+__device__ __forceinline__ bool x_maybe(int e, uint32_t least_v, const uint32_t (&x)[8]) {
+  const int room = e - 28 - x_exponent(least_v);
+  if (room <= -24) return false;
+  uint32_t m = 0xFFFFFFFFu;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) m = __vminu2(m, __vsub2(x[i] & 0x7FFF7FFFu, 0x00010001u));  // zeros wrap to the top
+  return room > x_exponent(min(m & 0xFFFFu, m >> 16) + 1u);
+}
+
+// Binade of a row's finite products (returned with 2 e + lacking: some pair lacks something), by a warp.
+__device__ __forceinline__ int x_scan(const XProblem& a, int ch, int m, int lane, bool* not_finite) {
+  float lmax = 0.f;
+  uint32_t lmin = 0xFFFFFFFFu;
+  bool inf = false;
+  x_products(a, ch, m, lane, [&](int, float p) {
+    lmin = min(lmin, x_mag(p) - 1u);  // zeros wrap to the top
+    if (x_mag(p) < kXInf) lmax = fmaxf(lmax, fabsf(p));
+    else inf = true;
+  });
+  const int e = x_binade(lmax);
+  *not_finite = __any_sync(0xffffffffu, inf);
+  return 2 * e + (__any_sync(0xffffffffu, inf || lmin < ((uint32_t)(127 - 28 + e) << 24) - 1u) ? 1 : 0);
+}
+// After batch row m of a chunk has been built: true when its pairs lack something. With infinities or NaN among the
+// products the row is built again, with the finite ones' factor and zeros in their places (layouts: x_build_row and
+// x_build_row2).
+template <bool BASE3, bool DIAG>
+__device__ __noinline__ bool x_search(const XProblem& a, int ch, int m, float* fold, const uint32_t* boff, uint8_t* bt) {
+  const int lane = x_lane();
+  bool not_finite;
+  const int es = x_scan(a, ch, m, lane, &not_finite);
+  if (!not_finite) return es & 1;
+  const float sc = x_sc(es >> 1);
+  const int q = lane >> 3, w = lane >> 2, n = BASE3 ? (DIAG ? 2 * q : 2 * (m & 3)) : (2 * (m & 3)) ^ (w & 3);
+  uint8_t* base = bt + (BASE3 ? (DIAG ? 8 * q : (m >> 2) * kXBTileBytes + 2048 * q)
+                              : (m >> 2) * kXTile2Bytes + w * 1024 + (lane & 3) * 8);
+  x_products(a, ch, m, lane, [&](int i, float p) {
+    uint32_t o = ((i & 7) >> 1) * 256 + 4 * (i & 1) + 2 * (i >> 3), col = (uint32_t)n;
+    if (BASE3) {
+      o = (boff[8 * (lane & 7) + (i >> 1)] >> (16 * (i & 1))) & 0xFFFFu;
+      col ^= o >> 14;
+      o = DIAG ? o & 0x3FFFu : (o & 0x1FFFu) + (o & 0x2000u ? 8192 - 2048 * q + 8 * q : 0);
+    }
+    __half2 hi, lo;
+    x_pair(x_mag(p) < kXInf ? p : 0.f, 0.f, sc, hi, lo);
+    *reinterpret_cast<__half*>(base + o + 32 * col) = __low2half(hi);
+    *reinterpret_cast<__half*>(base + o + 32 * (col ^ 1u)) = __low2half(lo);
+  });
+  if (lane == 0) fold[m] = x_fold(es >> 1);
+  return true;
+}
+
 // One batch row's B operand of a chunk, by one warp (lane = 16 columns; boff: the block's places, two
-// columns a word). DIAG (M =
+// columns a word). True when the lane's pairs may lack something. DIAG (M =
 // 1): column pair q of the tile for block q, else column pair m % 4. The factor 2^-E and the blocks'
 // sums of x go to fold[m] and sx[block][m].
 template <bool DIAG>
-__device__ __forceinline__ void x_build_row(const uint32_t (&x)[8], const uint32_t (&v)[8], int m, const uint32_t* boff, uint8_t* bt, float* fold,
-                                            float* sx, int lane) {
+__device__ __forceinline__ bool x_build_row(const uint32_t (&x)[8], const uint32_t (&v)[8], int m, const uint32_t* boff, uint8_t* bt, float* fold,
+                                            float* sx, uint32_t least_v, int lane) {
   // v*x is exact in fp32; formed here for the largest and again below (sixteen registers fewer)
-  auto product = [&](int i) {
-    return h2f((uint16_t)(v[i >> 1] >> (16 * (i & 1)))) * h2f((uint16_t)(x[i >> 1] >> (16 * (i & 1))));
-  };
-  float sum = 0.f, lmax = 0.f, probe = 0.f;
+  auto product = [&](int i) { return x_fma16(x_half(v[i >> 1], i & 1), x_half(x[i >> 1], i & 1), 0.f); };
+  float sum = 0.f, lmax = 0.f;
 #pragma unroll
   for (int i = 0; i < 16; ++i) {
-    const float p = product(i);
-    sum += h2f((uint16_t)(x[i >> 1] >> (16 * (i & 1))));
-    lmax = fmaxf(lmax, fabsf(p));
-    probe = fmaf(p, 0.f, probe);
+    sum = x_add16(x_half(x[i >> 1], i & 1), sum);
+    lmax = x_max_nan(lmax, fabsf(product(i)));
   }
-  // an infinity or NaN in v*x (fmaxf drops NaN) makes the row's result NaN
-  if (!(fabsf(probe) <= 1.f)) lmax = __int_as_float(0x7f800000);
-  const uint32_t amax = __reduce_max_sync(0xffffffffu, __float_as_uint(lmax));
-  const int e = amax ? (int)(amax >> 23) - 127 : 0;  // |v*x| < 2^(e + 1)
-  const float sc = __uint_as_float((uint32_t)(127 + 13 - e) << 23);  // half of 2^E, E = 14 - e
+  const int e = x_binade(lmax);
+  const float sc = x_sc(e);
+  if (lane == 0) fold[m] = x_fold(e);
   const int q = lane >> 3, n = DIAG ? 2 * q : 2 * (m & 3);  // the lane's block, the hi column
   uint8_t* tile = bt + (DIAG ? 8 * q : (m >> 2) * kXBTileBytes + 2048 * q);
   const int tail = 8192 - 2048 * q + 8 * q;  // from there: bytes 24 and 25
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    const float f0 = product(2 * i) * sc, f1 = product(2 * i + 1) * sc;
     const uint32_t ow = boff[8 * (lane & 7) + i];
-    const __half2 hi = __floats2half2_rn(f0, f1);
-    const __half2 lo = __floats2half2_rn(f0 - __low2float(hi), f1 - __high2float(hi));
+    __half2 hi, lo;
+    x_pair(product(2 * i), product(2 * i + 1), sc, hi, lo);
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       const uint32_t o = (ow >> (16 * k)) & 0xFFFFu;
@@ -270,7 +416,7 @@ __device__ __forceinline__ void x_build_row(const uint32_t (&x)[8], const uint32
   sum += __shfl_xor_sync(0xffffffffu, sum, 2);
   sum += __shfl_xor_sync(0xffffffffu, sum, 4);
   if ((lane & 7) == 0) sx[16 * q + m] = sum;
-  if (lane == 0) fold[m] = __uint_as_float((uint32_t)(127 - 14 + e) << 23);  // 2^-E
+  return x_maybe(e, least_v, x);
 }
 
 // 2-bit codes: one batch row's B operand of a chunk, by one warp. The lane's 16 columns are one code word, W =
@@ -279,43 +425,38 @@ __device__ __forceinline__ void x_build_row(const uint32_t (&x)[8], const uint32
 // with 4 (w & 3). Split: columns 2 (m % 4) and + 1 of tile m / 4 hold the fp16 pair whose sum is v*x 2^E / 2;
 // else column m % 8 of tile m / 8 holds x itself. SUM: the groups' sums of x too (for beta).
 template <bool SPLIT, bool SUM>
-__device__ __forceinline__ void x_build_row2(const uint32_t (&x)[8], const uint32_t (&v)[8], int m, uint8_t* bt, float* fold,
-                                             float* sx, int lane) {
+__device__ __forceinline__ bool x_build_row2(const uint32_t (&x)[8], const uint32_t (&v)[8], int m, uint8_t* bt, float* fold,
+                                             float* sx, uint32_t least_v, int lane) {
   const int q = lane & 3, w = lane >> 2, key = w & 3;
   float sum = 0.f;
   uint8_t* base = bt + (SPLIT ? m >> 2 : m >> 3) * kXTile2Bytes + w * 1024 + q * 8;
+  bool maybe = false;
   if constexpr (SPLIT) {
-    auto product = [&](int i) {  // exact in fp32
-      return h2f((uint16_t)(v[i >> 1] >> (16 * (i & 1)))) * h2f((uint16_t)(x[i >> 1] >> (16 * (i & 1))));
-    };
-    float lmax = 0.f, probe = 0.f;
+    auto product = [&](int i) { return x_fma16(x_half(v[i >> 1], i & 1), x_half(x[i >> 1], i & 1), 0.f); };
+    float lmax = 0.f;
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
-      const float p = product(i);
-      if (SUM) sum += h2f((uint16_t)(x[i >> 1] >> (16 * (i & 1))));
-      lmax = fmaxf(lmax, fabsf(p));
-      probe = fmaf(p, 0.f, probe);
+      if (SUM) sum = x_add16(x_half(x[i >> 1], i & 1), sum);
+      lmax = x_max_nan(lmax, fabsf(product(i)));
     }
-    if (!(fabsf(probe) <= 1.f)) lmax = __int_as_float(0x7f800000);  // an infinity or NaN makes the row NaN
-    const uint32_t amax = __reduce_max_sync(0xffffffffu, __float_as_uint(lmax));
-    const int e = amax ? (int)(amax >> 23) - 127 : 0;
-    const float sc = __uint_as_float((uint32_t)(127 + 13 - e) << 23);
+    const int e = x_binade(lmax);
+    const float sc = x_sc(e);
+    if (lane == 0) fold[m] = x_fold(e);
+    maybe = x_maybe(e, least_v, x);
     const int n = (2 * (m & 3)) ^ key;
 #pragma unroll
     for (int T = 0; T < 4; ++T) {
       uint32_t hi[2], lo[2];
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
-        const float f0 = product(2 * T + k) * sc, f1 = product(2 * T + k + 8) * sc;
-        const __half2 h = __floats2half2_rn(f0, f1);
-        const __half2 l = __floats2half2_rn(f0 - __low2float(h), f1 - __high2float(h));
+        __half2 h, l;
+        x_pair(product(2 * T + k), product(2 * T + k + 8), sc, h, l);
         hi[k] = *reinterpret_cast<const uint32_t*>(&h);
         lo[k] = *reinterpret_cast<const uint32_t*>(&l);
       }
       *reinterpret_cast<uint2*>(base + T * 256 + 32 * n) = make_uint2(hi[0], hi[1]);
       *reinterpret_cast<uint2*>(base + T * 256 + 32 * (n ^ 1)) = make_uint2(lo[0], lo[1]);
     }
-    if (lane == 0) fold[m] = __uint_as_float((uint32_t)(127 - 14 + e) << 23);  // 2^-E
   } else {
     const int n = (m & 7) ^ key;
     if (SUM) {
@@ -333,6 +474,7 @@ __device__ __forceinline__ void x_build_row2(const uint32_t (&x)[8], const uint3
     sum += __shfl_xor_sync(0xffffffffu, sum, 4);
     if ((lane & 7) == 0) sx[16 * (lane >> 3) + m] = sum;
   }
+  return maybe;
 }
 // v in the same order, [32 steps][4 lanes] 8-byte entries.
 __device__ __forceinline__ void x_build_v(const uint32_t (&v)[8], uint8_t* vt, int lane) {
@@ -553,8 +695,8 @@ __device__ __forceinline__ void x_decode_diag(const uint8_t* codes, int row_slot
   }
 #pragma unroll
   for (int k = 0; k < BLK; ++k) {
-    sum[k][0] = (acc[0][k][0] + acc[1][k][0]) + (acc[0][k][1] + acc[1][k][1]);
-    sum[k][1] = (acc[0][k][2] + acc[1][k][2]) + (acc[0][k][3] + acc[1][k][3]);
+    sum[k][0] = fmaf(acc[0][k][1] + acc[1][k][1], kXLo, acc[0][k][0] + acc[1][k][0]);
+    sum[k][1] = fmaf(acc[0][k][3] + acc[1][k][3], kXLo, acc[0][k][2] + acc[1][k][2]);
   }
 }
 
@@ -640,7 +782,7 @@ __device__ __forceinline__ void x_decode_rows(const uint8_t* row, int off, int r
       for (int j = 0; j < MT; ++j) {
         float& t = part[r >> 1][j][r & 1];
         const float* a2 = &acc[r >> 1][j][2 * (r & 1)];
-        t = fmaf(al, (a2[0] + a2[1]) * fold[4 * j + q], t);
+        t = fmaf(al, fmaf(a2[1], kXLo, a2[0]) * fold[4 * j + q], t);
         if (bias) t = fmaf(be, sx[16 * blk + 4 * j + q], t);
       }
     }
@@ -691,8 +833,8 @@ __device__ __forceinline__ void x_decode_rows(const uint8_t* row, int off, int r
 #pragma unroll
     for (int j = 0; j < MT; ++j) {
       const float F = fold[4 * j + q] * up;
-      run[k][j][0] += fmaf(acc[k][j][0] + acc[k][j][1], F, part[k][j][0]);
-      run[k][j][1] += fmaf(acc[k][j][2] + acc[k][j][3], F, part[k][j][1]);
+      run[k][j][0] += fmaf(fmaf(acc[k][j][1], kXLo, acc[k][j][0]), F, part[k][j][0]);
+      run[k][j][1] += fmaf(fmaf(acc[k][j][3], kXLo, acc[k][j][2]), F, part[k][j][1]);
     }
 }
 
@@ -786,7 +928,7 @@ __device__ __forceinline__ void x_decode2(const uint8_t* codes, const uint8_t* b
         const float *d = &acc[0][r >> 1][j][2 * (r & 1)], *e = &acc[1][r >> 1][j][2 * (r & 1)];
         if constexpr (SPLIT) {
           float& t = GRP ? part[r >> 1][j][r & 1] : run[r >> 1][j][r & 1];
-          const float sum = ((d[0] + e[0]) + (d[1] + e[1])) * fold[4 * j + q];
+          const float sum = fmaf(d[1] + e[1], kXLo, d[0] + e[0]) * fold[4 * j + q];
           if (GRP) t += fmaf(a1, sum, bias ? be * sx[16 * blk + 4 * j + q] : 0.f);
           else t = fmaf(a1, sum, t);
         } else {
@@ -808,6 +950,65 @@ __device__ __forceinline__ void x_decode2(const uint8_t* codes, const uint8_t* b
 #pragma unroll
         for (int z = 0; z < NV; ++z) run[k][j][z] += part[k][j][z];
   }
+}
+
+// What B lacks of batch row m in chunk ch: the sum of alpha T x_lacking(v*x) in fp32, and of the residual's values times
+// x where x is not finite, for the thread's rows row0, row0 + 8, + 16, + 24. Everything is read from global memory
+// again: two passes over the chunk to find the columns, some 500 cycles for each. Rare (an activation 2^28
+// times another one of its chunk).
+template <bool BASE3>
+__device__ __noinline__ float4 x_left_out(const XProblem& a, int ch, int m, int row0) {
+  constexpr int R = 2 * kXBlocks;
+  const int lane = x_lane();
+  const uint16_t* xm = a.x + (size_t)m * a.K;
+  bool not_finite;
+  const float sc = x_sc(x_scan(a, ch, m, lane, &not_finite) >> 1);
+  uint32_t mask = 0u;
+  x_products(a, ch, m, lane, [&](int i, float p) {
+    if (x_lacking(p, sc) != 0.f) mask |= 1u << i;  // a NaN too
+  });
+  float out[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) out[r] = 0.f;
+  for (uint32_t lanes; (lanes = __ballot_sync(0xffffffffu, mask != 0u)) != 0u;) {
+    const int src = __ffs((int)lanes) - 1;
+    const int k = ch * kXChunkCols + 16 * src + __ffs((int)__shfl_sync(0xffffffffu, mask, src)) - 1;
+    if (lane == src) mask &= mask - 1u;
+    const float p = x_lacking(h2f(__ldg(a.v + k)) * h2f(__ldg(xm + k)), sc);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int row = min(row0 + 8 * r, a.N - 1);  // rows past N: never written
+      const uint8_t* codes = a.packed + (size_t)row * a.row_bytes;
+      int T;
+      if (BASE3) {
+        int b = __ldg(codes + 26 * (k >> 7) + (k & 127) / 5);
+        for (int d = (k & 127) % 5; d > 0; --d) b /= 3;
+        T = b % 3 - 1;
+      } else {
+        T = ((__ldg(codes + (k >> 2)) >> (2 * (k & 3))) & 3) - 1;
+      }
+      const size_t g = a.G == 1 ? (size_t)row : (size_t)row * a.G + (k >> 7);
+      if (T) out[r] = fmaf(h2f(__ldg(a.scales + (a.bias ? 2 * g : g))), T > 0 ? p : -p, out[r]);
+    }
+  }
+  const int e = ch * (a.res_q * a.n_chunks + a.res_r), st0 = e / a.n_chunks;
+  const int n_steps = a.res_q + (e - st0 * a.n_chunks + a.res_r >= a.n_chunks ? 1 : 0);
+  uint16_t xs = 0;
+  if (x_has_sal(a, st0, n_steps, lane)) xs = x_at_sal(a, m, __ldg(a.sal + 16 * st0 + lane));
+  for (uint32_t lanes = __ballot_sync(0xffffffffu, !x_finite(xs)); lanes; lanes &= lanes - 1u) {
+    const int src = __ffs((int)lanes) - 1, c = 16 * st0 + src;
+    const float xe = h2f((uint16_t)__shfl_sync(0xffffffffu, (uint32_t)xs, src));
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int row = min(row0 + 8 * r, a.N - 1), grp = row >> 2;
+      if (((__ldg(a.ridx + (size_t)grp * ((a.s + 3) >> 2) + (c >> 2)) >> (2 * (c & 3))) & 3) != (row & 3)) continue;
+      const size_t i = (size_t)grp * a.s + c;
+      const uint16_t h = a.fp8 ? (uint16_t)x_e4m3x2(__ldg(reinterpret_cast<const uint8_t*>(a.rvals) + i))
+                               : __ldg(reinterpret_cast<const uint16_t*>(a.rvals) + i);
+      out[r] = fmaf(h2f(h), xe, out[r]);
+    }
+  }
+  return make_float4(out[0], out[1], out[2], out[3]);
 }
 
 // MT: n8 tiles of B (four batch rows each, eight with kXV2). GRP: alpha and beta staged per unit and 128-column
@@ -837,6 +1038,10 @@ __global__ void __launch_bounds__(kXThreads, 1)
     for (int i = threadIdx.x; i < NP * (int)(sizeof(XProblem) / 4); i += kXThreads) dst[i] = src[i];
   }
   uint2* mask = reinterpret_cast<uint2*>(boff + 64);                 // [256] x_mask
+  // batch rows with products left out of B, by chunk (chunk % kXOutWords: bits that a chunk does not need do no harm),
+  // then over all chunks
+  uint32_t* left_out = reinterpret_cast<uint32_t*>(mask + 256);
+  for (int i = threadIdx.x; i <= kXOutWords; i += kXThreads) left_out[i] = 0u;
   for (int i = threadIdx.x; i < 256; i += kXThreads) mask[i] = x_mask((uint32_t)i);
   if (BASE3 && threadIdx.x < 64)
     boff[threadIdx.x] = x_b_offset<DIAG>(2 * threadIdx.x) | x_b_offset<DIAG>(2 * threadIdx.x + 1) << 16;
@@ -934,19 +1139,44 @@ __global__ void __launch_bounds__(kXThreads, 1)
           *reinterpret_cast<uint32_t*>(sb + lay.rpos + 4 * ht) = pos.b[0] | pos.b[1] << 8 | pos.b[2] << 16 | pos.b[3] << 24;
       }
       x_cp_arrive(smem_u32(&full[st]));
+      const uint32_t least_v = VENC ? 0u : x_least(rows.v);
+      uint32_t maybe = 0u;  // bit m: the pairs of batch row m may lack something; bit 16 + m: some x at a salient column does
 #pragma unroll
       for (int k = 0; k < R; ++k) {
         const int m = hw + k * H;
         if (m >= M) break;
+        if (!VENC && rsn > 0) {
+          if (!x_finite(xs[k])) {
+            maybe |= 0x10000u << m;
+            xs[k] = 0;
+          }
+        }
         const int tile = VENC ? m >> 3 : m >> 2, n = VENC ? m & 7 : 2 * (m & 3);
         if (lane < 16 * rsn)  // x at the salient entries: the row's column, or the hi column of its pair
           *reinterpret_cast<uint16_t*>(sb + lay.rb + tile * kXResBBytes +
                                        ((lane >> 4) * 32 + 4 * n + ((lane >> 2) & 3)) * 8 + 2 * (lane & 3)) = xs[k];
         float* fold = reinterpret_cast<float*>(sb + lay.fold);
         float* sx = reinterpret_cast<float*>(sb + lay.sx);
-        if constexpr (BASE3) x_build_row<DIAG>(rows.x[k], rows.v, m, boff, sb + lay.b, fold, sx, lane);
-        else x_build_row2<!VENC, GRP>(rows.x[k], rows.v, m, sb + lay.b, fold, sx, lane);
+        bool lacks;
+        if constexpr (BASE3) lacks = x_build_row<DIAG>(rows.x[k], rows.v, m, boff, sb + lay.b, fold, sx, least_v, lane);
+        else lacks = x_build_row2<!VENC, GRP>(rows.x[k], rows.v, m, sb + lay.b, fold, sx, least_v, lane);
+        if (lacks) maybe |= 1u << m;
         if (VENC && m == 0) x_build_v(rows.v, sb + lay.v, lane);
+      }
+      if constexpr (!VENC) {
+        maybe = __reduce_or_sync(0xffffffffu, maybe);
+        if (maybe) {
+          uint32_t rows_out = maybe >> 16;
+          for (uint32_t rest = maybe & 0xFFFFu; rest; rest &= rest - 1u) {
+            const int m = __ffs((int)rest) - 1;
+            if (x_search<BASE3, DIAG>(a, c.ch, m, reinterpret_cast<float*>(sb + lay.fold), boff, sb + lay.b))
+              rows_out |= 1u << m;
+          }
+          if (rows_out && lane == 0) {
+            atomicOr(left_out + (c.ch & (kXOutWords - 1)), rows_out);
+            atomicOr(left_out + kXOutWords, rows_out);
+          }
+        }
       }
       mbar_arrive(smem_u32(&full[st]));
       c = n1;
@@ -1009,7 +1239,7 @@ __global__ void __launch_bounds__(kXThreads, 1)
       const int o0 = off + 26 * q;
       float sum[BLK][2];
       x_decode_diag<BLK>(row + (o0 & ~3), row_slot, 8 * (o0 & 2), sb + lay.b, lane, sum);
-      const float F = fold[0], bx = sx[16 * q];
+      const float F = fold[0], bx = a.bias ? sx[16 * q] : 0.f;
 #pragma unroll
       for (int r = 0; r < 2 * BLK; ++r) {
         const uint32_t ab = *reinterpret_cast<const uint32_t*>(sc + r * 128 + 4 * q);
@@ -1040,6 +1270,22 @@ __global__ void __launch_bounds__(kXThreads, 1)
 
     if (c.ch == cur.n_chunks - 1 || u == u1 - 1) {
       // ---- the tile's epilogue once this CTA's part of it is done
+      const int A = a.unit_begin + c.t * a.n_chunks, B = A + a.n_chunks;
+      if (!VENC && __any_sync(0xffffffffu, left_out[kXOutWords] != 0u)) {
+        for (int ch = max(u0 - A, 0); ch <= c.ch; ++ch) {
+          // read once for the warp: the helpers may be adding bits for later units
+          uint32_t rows_out = __shfl_sync(0xffffffffu, left_out[ch & (kXOutWords - 1)], 0);
+          for (; rows_out; rows_out &= rows_out - 1u) {
+            const int m = __ffs((int)rows_out) - 1;
+            const float4 o4 = x_left_out<BASE3>(a, ch, m, c.t * kXTileRows + tr + g);
+            const float add[4] = {o4.x, o4.y, o4.z, o4.w};
+#pragma unroll
+            for (int j = 0; j < MT; ++j)
+#pragma unroll
+              for (int r = 0; r < 2 * BLK; ++r) run[r >> 1][j][r & 1] += 4 * j + q == m ? add[r] : 0.f;
+          }
+        }
+      }
       if (DIAG) {  // the four blocks' shares, in lane order
 #pragma unroll
         for (int k = 0; k < BLK; ++k)
@@ -1049,7 +1295,6 @@ __global__ void __launch_bounds__(kXThreads, 1)
             run[k][0][h] += __shfl_xor_sync(0xffffffffu, run[k][0][h], 2);
           }
       }
-      const int A = a.unit_begin + c.t * a.n_chunks, B = A + a.n_chunks;
       constexpr int kWords = BLK * MT * NV;
       bool write = true;
       if (A < u0) {
