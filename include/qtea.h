@@ -150,9 +150,9 @@ int qtea_pack_layout(const int8_t* ternary_codes, int N, int K, int group_size, 
  * tensor-core kernel 2T and v*x are exact (v*x as an fp16 pair down to 2^-28 of the largest of its 512
  * columns, what smaller products lack of it added in fp32), products are summed on the tensor cores over at most
  * 512 columns, the rest in fp32 (a column where v*x is infinite or NaN counts in the rows whose code there is not 0,
- * or that hold its residual value); 2-bit layouts at M >= 5, and the older low-batch
- * kernel, take 2T*v and x in fp16 (both exact, which needs |v| < 32768; an infinity or NaN in x makes the batch row
- * NaN). On the fixed-point
+ * or that hold its residual value); 2-bit layouts at M >= 5 take 2T*v and x in fp16 there, both exact, and where
+ * that gives no finite sum (|v| >= 32768, infinities and NaN) the sum is formed in fp32. The older low-batch
+ * kernel takes 2T*v and x in fp16 too, which needs |v| < 32768; an infinity or NaN in x makes the batch row NaN. On the fixed-point
  * kernel (when v*x of the call fits in shared memory): the ternary sum is accumulated exactly in integers over 128-column blocks, with v*x in fixed point relative to the
  * block's largest |v*x| (|X| < 2^23) after up to 3 massive values per block are taken out and
  * added exactly in fp32; block sums, alpha, beta and the residual are combined in fp32. Other

@@ -19,7 +19,8 @@
 //    and NaN are added in fp32 at the end of the tile, to the rows whose code there is not 0. Four batch
 //    rows make one n8 tile. The sums are folded with 2^-E per chunk. 2-bit codes at
 //    M >= 5 have v in A instead (2T * v, one exact fp16 multiply) and x in B, eight batch rows to a tile: half the
-//    MMAs (at M = 16 the decoding loop alone runs at 38 weights per clock per SM, with four split tiles at 27).
+//    MMAs (at M = 16 the decoding loop alone runs at 38 weights per clock per SM, with four split tiles at 27). From
+//    |v| = 2^15 on, and for infinities and NaN in x, the tile's batch row is done again in fp32.
 //  * Scales: base-3 at M = 1: column pair q of the tile is non-zero only in the k slots of lane q, so that a
 //    thread's accumulators hold its own block's sums; at M >= 2 the accumulators are folded per block (2-bit with
 //    one scale per row: per unit). Either way alpha, and beta times the block's sum of x, are applied in fp32 (but
@@ -1011,6 +1012,58 @@ __device__ __noinline__ float4 x_left_out(const XProblem& a, int ch, int m, int 
   return make_float4(out[0], out[1], out[2], out[3]);
 }
 
+// Batch row m over chunks ch0 .. ch1 with v in A, done again in fp32 as the general kernels do, for the thread's rows row0,
+// row0 + 8, + 16, + 24 (the quad's lanes take every fourth column and salient entry). For tiles that came out
+// infinite or NaN: from |v| = 2^15 on 2v is no fp16 number, and an infinity or NaN in x meets every row through 0 *
+// x; here it counts in the rows whose code, or residual position, it meets. Found by looking at the tile's sums, which
+// costs nothing (looking at x and v as they are staged: Qwen3-14B layer, M = 16, 53.2 -> 54.7 us).
+__device__ __noinline__ float4 x_again(const XProblem& a, int ch0, int ch1, int m, int row0) {
+  constexpr int R = 2 * kXBlocks;
+  const int q = x_lane() & 3;
+  const uint16_t* xm = a.x + (size_t)m * a.K;
+  const uint8_t* codes[R];
+  const uint16_t* scales[R];
+  float out[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int row = min(row0 + 8 * r, a.N - 1);  // rows past N: never written
+    codes[r] = a.packed + (size_t)row * a.row_bytes;
+    scales[r] = a.scales + (size_t)row * a.G * (a.bias ? 2 : 1);
+    out[r] = 0.f;
+  }
+  for (int k = ch0 * kXChunkCols + q; k < min(a.K, (ch1 + 1) * kXChunkCols); k += 4) {
+    const uint16_t xk = __ldg(xm + k);
+    const float p = x_fma16(__ldg(a.v + k), xk, 0.f);
+    const int g = a.G == 1 ? 0 : k >> 7;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int T = ((__ldg(codes[r] + (k >> 2)) >> (2 * (k & 3))) & 3) - 1;
+      if (T) out[r] = fmaf(h2f(__ldg(scales[r] + (a.bias ? 2 * g : g))), T > 0 ? p : -p, out[r]);
+      if (a.bias) out[r] = fmaf(h2f(__ldg(scales[r] + 2 * g + 1)), h2f(xk), out[r]);
+    }
+  }
+  const int per = a.res_q * a.n_chunks + a.res_r;  // the chunks' salient entries: steps [ch0 per / n, (ch1 + 1) per / n)
+  const int c1 = min(a.s, 16 * (int)((long long)(ch1 + 1) * per / a.n_chunks));
+  for (int c = 16 * (ch0 * per / a.n_chunks) + q; c < c1; c += 4) {
+    const float xc = h2f(x_at_sal(a, m, __ldg(a.sal + c)));
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int row = min(row0 + 8 * r, a.N - 1), grp = row >> 2;
+      if (((__ldg(a.ridx + (size_t)grp * ((a.s + 3) >> 2) + (c >> 2)) >> (2 * (c & 3))) & 3) != (row & 3)) continue;
+      const size_t i = (size_t)grp * a.s + c;
+      const uint16_t h = a.fp8 ? (uint16_t)x_e4m3x2(__ldg(reinterpret_cast<const uint8_t*>(a.rvals) + i))
+                               : __ldg(reinterpret_cast<const uint16_t*>(a.rvals) + i);
+      out[r] = fmaf(h2f(h), xc, out[r]);
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    out[r] += __shfl_xor_sync(0xffffffffu, out[r], 1);
+    out[r] += __shfl_xor_sync(0xffffffffu, out[r], 2);
+  }
+  return make_float4(out[0], out[1], out[2], out[3]);
+}
+
 // MT: n8 tiles of B (four batch rows each, eight with kXV2). GRP: alpha and beta staged per unit and 128-column
 // group (always with base-3 codes), else one alpha per row.
 template <int MT, int MODE, bool GRP>
@@ -1271,7 +1324,31 @@ __global__ void __launch_bounds__(kXThreads, 1)
     if (c.ch == cur.n_chunks - 1 || u == u1 - 1) {
       // ---- the tile's epilogue once this CTA's part of it is done
       const int A = a.unit_begin + c.t * a.n_chunks, B = A + a.n_chunks;
-      if (!VENC && __any_sync(0xffffffffu, left_out[kXOutWords] != 0u)) {
+      if constexpr (VENC) {
+        uint32_t again = 0u;  // batch rows with a sum that is not finite
+#pragma unroll
+        for (int j = 0; j < MT; ++j)
+#pragma unroll
+          for (int z = 0; z < 2; ++z) {
+            float f = 0.f;
+#pragma unroll
+            for (int r = 0; r < 2 * BLK; ++r) f = fmaf(run[r >> 1][j][2 * (r & 1) + z], 0.f, f);
+            if (f != 0.f) again |= 1u << (8 * j + 2 * q + z);
+          }
+        again = __reduce_or_sync(0xffffffffu, again) & ((1u << M) - 1u);
+        for (; again; again &= again - 1u) {
+          const int m = __ffs((int)again) - 1;
+          const float4 s4 = x_again(a, max(u0 - A, 0), c.ch, m, c.t * kXTileRows + tr + g);
+          const float sum[4] = {s4.x, s4.y, s4.z, s4.w};
+#pragma unroll
+          for (int j = 0; j < MT; ++j)
+#pragma unroll
+            for (int z = 0; z < 2; ++z)
+              if (8 * j + 2 * q + z == m)
+#pragma unroll
+                for (int r = 0; r < 2 * BLK; ++r) run[r >> 1][j][2 * (r & 1) + z] = sum[r];
+        }
+      } else if (__any_sync(0xffffffffu, left_out[kXOutWords] != 0u)) {
         for (int ch = max(u0 - A, 0); ch <= c.ch; ++ch) {
           // read once for the warp: the helpers may be adding bits for later units
           uint32_t rows_out = __shfl_sync(0xffffffffu, left_out[ch & (kXOutWords - 1)], 0);

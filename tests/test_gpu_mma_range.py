@@ -1,7 +1,8 @@
 """Activations of a wide range on the tensor-core kernel with staged B operands, against the fp64 oracle: one massive
 value per 512-column chunk beside activations down to 2^-36 of it, with codes 0 at the massive columns in part of
 the rows, where an error relative to the massive value shows. v*x is held as an fp16 pair, exact down to 2^-28 of
-the chunk's largest; what smaller products lack of it is added in fp32, as infinities and NaN are.
+the chunk's largest; what smaller products lack of it is added in fp32, as infinities and NaN are. (2-bit codes at M
+>= 5 take 2T v in A instead, exact below |v| = 2^15; larger v are added in fp32 too.)
 
 Pass rule per element: |y - y_ref| <= 2e-6 * sum_j |x_j * W^[o][j]|, nothing absolute. Every product is exact; the
 tensor core truncates each of a chunk's at most 35 steps below 2^-24 of the partial sum, and what the pairs lack (up
@@ -89,7 +90,7 @@ def test_spread_over_every_binade(qt, fmt, M):
     assert np.all(err <= REL * bound), f"worst {(err / bound).max():.3g} of the bound"
 
 
-@pytest.mark.parametrize("fmt,M", [f for f in FORMS if f[0] == "base3" or f[1] <= 4])
+@pytest.mark.parametrize("fmt,M", FORMS)
 @pytest.mark.parametrize("group,bias", [(0, False), (128, False)])
 def test_infinities_and_nan_reach_their_rows_only(qt, fmt, M, group, bias):
     """A column whose activation is infinite or NaN counts in the rows with a non-zero code (or a residual value)
@@ -122,6 +123,23 @@ def test_infinities_and_nan_reach_their_rows_only(qt, fmt, M, group, bias):
     assert np.array_equal(y[~ok], special[~ok], equal_nan=True)
     assert np.all(np.abs(y - y_ref)[ok] <= REL * bound[ok])
     assert ok.sum() > M * N / 8 and (~ok).sum() > 0
+
+
+@pytest.mark.parametrize("fmt,M", FORMS + [("2bit", 5), ("2bit", 9)])
+@pytest.mark.parametrize("group,bias", [(0, False), (0, True), (128, True)])
+def test_column_scales_of_any_size(qt, fmt, M, group, bias):
+    """|v| from fp16's smallest to its largest (2 v is no fp16 number from 2^15 on)."""
+    N, K, fp8 = 132, 1100, fmt == "2bit" and M == 1
+    p = synth.make_problem("v", N, K, M, 24, seed=11 + M, group_size=group, beta_std=0.002 if bias else 0.0, residual_fp8=fp8)
+    v = p.v.view(np.float16)
+    v[5::97] = 65504.0
+    v[6::97] = -32768.0
+    v[7::97] = 32752.0
+    v[8::97] = 2.0 ** -24
+    y_ref, bound = oracle.gemv(p.x, p.T, p.alpha, p.v, p.salient_idx, p.residual_vals, p.residual_idx,
+                               beta=p.beta if bias else None, group_size=group or K, residual_fp8=fp8)
+    err = np.abs(call(qt, p, fmt, bias, fp8) - y_ref)
+    assert np.all(err <= REL * bound), f"worst {(err / bound).max():.3g} of the bound"
 
 
 def oracle_value(p, k, fp8):
