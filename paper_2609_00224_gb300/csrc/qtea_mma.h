@@ -493,7 +493,10 @@ __device__ __forceinline__ void x_stage_scales(const XProblem& a, const XPos& c,
 #pragma unroll
   for (int k = 0; k < kXTileRows / (32 * H); ++k) {
     const int r = ht + k * 32 * H, row = c.t * kXTileRows + r;
-    if (row >= a.N) break;
+    if (row >= a.N) {  // zero: their alphas take part in the warp's votes
+      *reinterpret_cast<uint4*>(dst + r * 16) = make_uint4(0u, 0u, 0u, 0u);
+      continue;
+    }
     if (a.scales_vec && a.bias) {
       x_cp16(smem_u32(dst + r * 16), a.scales + 2 * ((size_t)row * a.G + 4 * c.ch));
       continue;
@@ -701,14 +704,19 @@ __device__ __forceinline__ void x_decode_diag(const uint8_t* codes, int row_slot
   }
 }
 
+// Alphas (fp16 bits) whose 2T alpha could be infinite, and those that may not be divided by 4.
+__device__ __forceinline__ bool x_big(uint32_t h) { return (h & 0x7FFFu) >= 0x7400u; }
+__device__ __forceinline__ bool x_tiny(uint32_t h) { return (h & 0x7FFFu) - 1u < 0x0C00u - 1u; }  // below 2^-12, not 0
+
 // M >= 2: the unit's 35 steps. The four lanes share each block (six bytes each, one accumulation of eight
 // steps, scaled by the rows' alpha in fp32: run += alpha_b 2^-E sum + beta_b sum_b(x)); the blocks' last
-// two bytes go to one lane each and carry alpha in A (a sixteenth of the columns, three steps). row: the
+// two bytes go to one lane each and carry alpha in A (a sixteenth of the columns, three steps; tiny: the lane has
+// alphas there that are left out). row: the
 // offset of the thread's first row in the stage; off: of the unit in the row.
 template <int MT, int BLK>
 __device__ __forceinline__ void x_decode_rows(const uint8_t* row, int off, int row_slot, const uint8_t* bt,
                                               const uint8_t* sc, const float* fold, const float* sx, bool bias,
-                                              int q, int lane, float (&run)[BLK][MT][2]) {
+                                              int q, int lane, bool& tiny, float (&run)[BLK][MT][2]) {
   constexpr int R = 2 * BLK;
   const int stride = 8 * row_slot;
   // the unit's sum on its own before it joins the tile's: 28 additions in a row instead of 112 for K = 14336
@@ -788,19 +796,23 @@ __device__ __forceinline__ void x_decode_rows(const uint8_t* row, int off, int r
       }
     }
   }
-  // bytes 24 and 25 of block q; alpha * 2T must stay finite: rows with some |alpha| >= 2^14 take alpha / 4
+  // bytes 24 and 25 of block q; alpha * 2T must stay finite: with some |alpha| >= 2^14 the warp takes alpha / 4, but for
+  // alphas that could lose bits that way (x_tiny), which are added at the end of the tile (x_left_out)
   uint32_t al[R];
   bool big = false;
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     al[r] = __byte_perm(*reinterpret_cast<const uint32_t*>(sc + r * 128 + 4 * q), 0u, 0x1010);
-    big = big || (al[r] & 0x7FFFu) >= 0x7400u;
+    big = big || x_big(al[r]);
   }
   float up = 1.f;
   if (__any_sync(0xffffffffu, big)) {
     up = 4.f;
 #pragma unroll
-    for (int r = 0; r < R; ++r) al[r] = x_hmul2(al[r], 0x34003400u);
+    for (int r = 0; r < R; ++r) {
+      tiny = tiny || x_tiny(al[r]);
+      al[r] = x_tiny(al[r]) ? 0u : x_hmul2(al[r], 0x34003400u);
+    }
   }
   XDigits<false> y[R];
   const int o0 = off + 26 * q + 24;
@@ -957,7 +969,7 @@ __device__ __forceinline__ void x_decode2(const uint8_t* codes, const uint8_t* b
 // x where x is not finite, for the thread's rows row0, row0 + 8, + 16, + 24. Everything is read from global memory
 // again: two passes over the chunk to find the columns, some 500 cycles for each. Rare (an activation 2^28
 // times another one of its chunk).
-template <bool BASE3>
+template <bool BASE3, bool DIAG>
 __device__ __noinline__ float4 x_left_out(const XProblem& a, int ch, int m, int row0) {
   constexpr int R = 2 * kXBlocks;
   const int lane = x_lane();
@@ -990,6 +1002,35 @@ __device__ __noinline__ float4 x_left_out(const XProblem& a, int ch, int m, int 
       }
       const size_t g = a.G == 1 ? (size_t)row : (size_t)row * a.G + (k >> 7);
       if (T) out[r] = fmaf(h2f(__ldg(a.scales + (a.bias ? 2 * g : g))), T > 0 ? p : -p, out[r]);
+    }
+  }
+  if (BASE3 && !DIAG) {  // the last two bytes of block q where x_decode_rows left them out
+    const int blk = 4 * ch + (lane & 3);
+    uint16_t al[R];
+    bool big = false;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int row = row0 + 8 * r;
+      const size_t g = a.G == 1 ? (size_t)row : (size_t)row * a.G + blk;
+      al[r] = row < a.N && blk < a.n_blocks ? __ldg(a.scales + (a.bias ? 2 * g : g)) : (uint16_t)0;
+      big = big || x_big(al[r]);
+    }
+    if (__any_sync(0xffffffffu, big)) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        float sum = 0.f;
+        if (x_tiny(al[r])) {
+          const uint8_t* codes = a.packed + (size_t)(row0 + 8 * r) * a.row_bytes + 26 * blk;
+          int b = __ldg(codes + 24) + 243 * __ldg(codes + 25);
+          for (int k = 128 * blk + 120; k < min(a.K, 128 * blk + 128); ++k, b /= 3) {
+            const float p = x_fma16(__ldg(a.v + k), __ldg(xm + k), 0.f);
+            if (x_mag(p) < kXInf) sum = fmaf((float)(b % 3 - 1), p - x_lacking(p, sc), sum);  // what B holds of it
+          }
+        }
+        sum *= h2f(al[r]);
+        sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+        out[r] += sum + __shfl_xor_sync(0xffffffffu, sum, 2);
+      }
     }
   }
   const int e = ch * (a.res_q * a.n_chunks + a.res_r), st0 = e / a.n_chunks;
@@ -1299,7 +1340,12 @@ __global__ void __launch_bounds__(kXThreads, 1)
         run[r >> 1][0][r & 1] += fmaf(h2f((uint16_t)ab), sum[r >> 1][r & 1] * F, h2f((uint16_t)(ab >> 16)) * bx);
       }
     } else {
-      x_decode_rows<MT, BLK>(row, off, row_slot, sb + lay.b, sc, fold, sx, a.bias != 0, q, lane, run);
+      bool tiny = false;
+      x_decode_rows<MT, BLK>(row, off, row_slot, sb + lay.b, sc, fold, sx, a.bias != 0, q, lane, tiny, run);
+      if (tiny) {
+        atomicOr(left_out + (c.ch & (kXOutWords - 1)), (1u << M) - 1u);
+        atomicOr(left_out + kXOutWords, 1u);
+      }
     }
     if (rsn > 0) {
       float acc[BLK][MT][4];
@@ -1354,7 +1400,7 @@ __global__ void __launch_bounds__(kXThreads, 1)
           uint32_t rows_out = __shfl_sync(0xffffffffu, left_out[ch & (kXOutWords - 1)], 0);
           for (; rows_out; rows_out &= rows_out - 1u) {
             const int m = __ffs((int)rows_out) - 1;
-            const float4 o4 = x_left_out<BASE3>(a, ch, m, c.t * kXTileRows + tr + g);
+            const float4 o4 = x_left_out<BASE3, DIAG>(a, ch, m, c.t * kXTileRows + tr + g);
             const float add[4] = {o4.x, o4.y, o4.z, o4.w};
 #pragma unroll
             for (int j = 0; j < MT; ++j)

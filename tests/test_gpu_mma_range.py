@@ -148,3 +148,24 @@ def oracle_value(p, k, fp8):
     if not fp8:
         return r.view(np.float16).astype(np.float64)
     return torch.from_numpy(np.ascontiguousarray(r)).view(torch.float8_e4m3fn).double().numpy()
+
+
+@pytest.mark.parametrize("fmt,M", [("base3", 2), ("base3", 5), ("base3", 16), ("2bit", 3), ("2bit", 12)])
+@pytest.mark.parametrize("massive", [False, True])
+def test_row_scales_far_apart(qt, fmt, M, massive):
+    """|alpha| of 30000, 1e-4, 2^-24 and 0 in neighbouring rows and groups: the small ones keep every bit, also where
+    activations of 2^-21 stand beside one of 6e4."""
+    N, K = 132, 700
+    p = synth.make_problem("alpha", N, K, M, 0, seed=21 + M, group_size=128, x_std=2.0 ** -21 if massive else 1.0)
+    if massive:
+        synth.plant_massive(p.x, M, [6e4], lo=0, hi=100)
+        synth.plant_massive(p.x, M, [6e4], lo=600, hi=700)
+    alpha = p.alpha.view(np.float16)
+    alpha[1::5] = 1e-4
+    alpha[2::5] = 2.0 ** -24
+    alpha[3::5] = 30000.0
+    alpha[3::10, 1] = 1.2e-4
+    alpha[4::10] = 0.0
+    y_ref, bound = oracle.gemv(p.x, p.T, p.alpha, p.v, p.salient_idx, p.residual_vals, p.residual_idx, group_size=128)
+    err = np.abs(call(qt, p, fmt, False, False) - y_ref)
+    assert np.all(err <= REL * bound), f"worst {np.nanmax(err / np.maximum(bound, 1e-30)):.3g} of the bound"
