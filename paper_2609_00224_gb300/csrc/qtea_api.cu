@@ -109,6 +109,7 @@ int plan_m1(qtea_layout* l, const cudaDeviceProp& prop, cudaStream_t st) {
                mb_prep_configure(prop.sharedMemPerBlockOptin) == cudaSuccess;
     l->prep_smem_optin = prop.sharedMemPerBlockOptin;
     l->mma2_ok = l->mb_ok && x_shape_ok(l, prop) && x_smem_bytes(3, 2, kChunkRowBytes, 2) <= prop.sharedMemPerBlockOptin &&
+                 x_smem_bytes(2, 4, kChunkRowBytes, 2) <= prop.sharedMemPerBlockOptin &&
                  mma2_configure(prop.sharedMemPerBlockOptin) == cudaSuccess;
     if (!l->mb_ok || !l->mma2_ok) cudaGetLastError();
     l->mb_smem_optin = mb_dyn;
@@ -258,12 +259,37 @@ bool mma2_eligible(const qtea_layout* l) { return l->mma2_ok && l->format == QTE
 // Scales staged per unit: groups of 128 columns, or beta.
 bool mma2_grp(const qtea_layout* l) { return l->group_size != l->K || (l->options & QTEA_OPT_BIAS); }
 
+// 2-bit codes at M >= 5 run with v in A, whose products of 22 bits the tensor core truncates: errors of 1.1e-7 to
+// 1.2e-7 of the outputs' norm with scale groups, as the older low-batch kernel's. Calls which that kernel does not take
+// (one alpha and beta per row; scale maps that are not whole aligned 16-byte vectors; FP8 residuals at odd
+// addresses) ran with fp32 sums, 0.75e-7 to 0.94e-7 at K <= 1152, and take the split form, 0.4e-7 to 0.9e-7, at 5 to 20 %
+// more time (K = 768, N = 4096, M = 16: 11.4 us with v in A, 13.2 split, 74 on the general kernel).
+bool mma2_split(const qtea_gemv_problem& q, int M) {
+  const qtea_layout* l = q.packed_ternary;
+  if (M <= 4) return false;
+  const bool bias = l->options & QTEA_OPT_BIAS;
+  if (l->group_size == l->K) {
+    if (bias) return true;
+  } else if (!aligned(q.row_scale, 16) || (l->K + 127) / 128 * (bias ? 4 : 2) % 16 != 0) {
+    return true;
+  }
+  return (l->options & QTEA_OPT_RESIDUAL_FP8) && l->n_salient > 0 &&
+         !(aligned(q.residual_vals, 16) && aligned(q.residual_idx, 16));
+}
+
 // Problems of the tensor-core kernel with staged B operands, of one format: up to kMaxProblems per launch
-// (2-bit ones with and without staged scales in launches of their own).
+// (2-bit ones with and without staged scales, and split ones at M >= 5, in launches of their own).
 int run_mma(const qtea_gemv_problem* qs, const int* idx, int n, bool base3, int M, cudaStream_t st) {
+  // with one split problem among them, those with scale groups or beta run split too: a launch fewer (7792x512, 140x1536
+  // and 280x1092 in one call, M = 9: 11.5 us in one launch, 21.4 in two)
+  bool any_split = false;
+  for (int i = 0; i < n && !base3; ++i) any_split = any_split || mma2_split(qs[idx[i]], M);
+  auto split_of = [&](const qtea_gemv_problem& q) {
+    return any_split && (mma2_grp(q.packed_ternary) || mma2_split(q, M));
+  };
   for (int i = 0; i < n;) {
     const qtea_layout* l0 = qs[idx[i]].packed_ternary;
-    const bool grp = base3 || mma2_grp(l0);
+    const bool split = split_of(qs[idx[i]]), grp = base3 || split || mma2_grp(l0);
     XParams P;
     std::memset(&P, 0, sizeof(P));
     P.M = M;
@@ -279,7 +305,7 @@ int run_mma(const qtea_gemv_problem* qs, const int* idx, int n, bool base3, int 
       const qtea_gemv_problem& q = qs[idx[i + k]];
       const qtea_layout* l = q.packed_ternary;
       if (l->sm_count != l0->sm_count) break;  // the partial rows are sized by the SM count
-      if (!base3 && mma2_grp(l) != grp) break;
+      if (!base3 && (split_of(q) || mma2_grp(l)) != grp) break;
       XProblem& a = P.prob[k];
       a.x = q.x;
       a.packed = l->packed;
@@ -317,7 +343,7 @@ int run_mma(const qtea_gemv_problem* qs, const int* idx, int n, bool base3, int 
     }
     P.n_problems = k;
     P.total_units = (int)units;
-    const int mode = x_mode(base3, M), mt = x_mt(mode, M);
+    const int mode = x_mode(base3, M, split), mt = x_mt(mode, M);
     int S = kXMaxStages;
     while (S > 2 && x_smem_bytes(mode, mt, P.row_slot, S) > l0->x_smem_optin) --S;
     P.n_stages = S;
@@ -326,7 +352,7 @@ int run_mma(const qtea_gemv_problem* qs, const int* idx, int n, bool base3, int 
     P.unit_q = (int)(units / grid);
     P.unit_r = (int)(units % grid);
     const size_t smem = x_smem_bytes(mode, mt, P.row_slot, S);
-    if ((base3 ? launch_b3mma(maps, P, grid, smem, st) : launch_mma2(maps, P, grp, grid, smem, st)) != cudaSuccess)
+    if ((base3 ? launch_b3mma(maps, P, grid, smem, st) : launch_mma2(maps, P, grp, split, grid, smem, st)) != cudaSuccess)
       return QTEA_ERR_CUDA;
     i += k;
   }

@@ -14,7 +14,7 @@ cudaError_t b3mma_configure(size_t smem_optin) {
 
 cudaError_t launch_b3mma(const TensorMaps& maps, const XParams& p, int grid, size_t smem, cudaStream_t st) {
   if (p.M == 1) return x_launch<1, kXDiag, true>(maps, p, grid, smem, st);
-  switch (x_mt(x_mode(true, p.M), p.M)) {
+  switch (x_mt(x_mode(true, p.M, true), p.M)) {
     case 1: return x_launch<1, kXRows, true>(maps, p, grid, smem, st);
     case 2: return x_launch<2, kXRows, true>(maps, p, grid, smem, st);
     case 3: return x_launch<3, kXRows, true>(maps, p, grid, smem, st);

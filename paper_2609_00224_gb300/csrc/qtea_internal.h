@@ -379,7 +379,9 @@ constexpr int kXBlocks = 2;                                    // 16-row blocks 
 constexpr int kXSets = 2;                                      // helper sets
 constexpr int kXThreads = 32 * (kXTileRows / 16 / kXBlocks + kXSets * kXHelpers);
 // Forms (XMode in qtea_mma.h) and n8 tiles.
-__host__ __device__ constexpr int x_mode(bool base3, int M) { return base3 ? (M == 1 ? 0 : 1) : (M <= 4 ? 2 : 3); }
+__host__ __device__ constexpr int x_mode(bool base3, int M, bool split) {
+  return base3 ? (M == 1 ? 0 : 1) : (M <= 4 || split ? 2 : 3);
+}
 __host__ __device__ constexpr int x_mt(int mode, int M) { return mode == 3 ? (M + 7) / 8 : (M + 3) / 4; }
 struct XStage {  // byte offsets within a stage; the codes start it
   int scales, rvals, rpos, b, rb, v, fold, sx, b_end, total;
@@ -439,7 +441,8 @@ inline size_t x_smem_bytes(int mode, int mt, int row_slot, int n_stages) {
 cudaError_t b3mma_configure(size_t smem_optin);
 cudaError_t launch_b3mma(const TensorMaps& maps, const XParams& p, int grid, size_t smem, cudaStream_t st);
 cudaError_t mma2_configure(size_t smem_optin);
-cudaError_t launch_mma2(const TensorMaps& maps, const XParams& p, bool grp, int grid, size_t smem, cudaStream_t st);
+cudaError_t launch_mma2(const TensorMaps& maps, const XParams& p, bool grp, bool split, int grid, size_t smem,
+                        cudaStream_t st);
 
 // ---------------------------------------------------------------- generic kernel (any M)
 struct GenericParams {

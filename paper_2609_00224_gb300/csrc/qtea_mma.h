@@ -63,7 +63,7 @@ namespace qtea {
 namespace {
 
 // The kernel's forms: base-3 codes at M = 1 and M >= 2, 2-bit codes with v*x split in two fp16 columns
-// per batch row (M <= 4) and with v in A and x in B (M >= 5).
+// per batch row (M <= 4, and where the launch asks for it) and with v in A and x in B (M >= 5).
 enum XMode { kXDiag = 0, kXRows = 1, kXSplit2 = 2, kXV2 = 3 };
 
 
@@ -895,27 +895,21 @@ constexpr int kXFoldV = 2;
 // at segment w ^ (row % 8)). SPLIT: B holds (hi, lo) of v*x 2^E / 2, folded with 2^-E; else A = 2T * v, one exact
 // fp16 multiply by the pairs in vt, and B holds x. GRP: the accumulators are folded per 128-column group with
 // the rows' alpha and beta of the group (staged at sc), else per unit with the row's alpha (al); with v in A,
-// whose products have 22 bits, two or four times a unit. run: [block]
+// whose products have 22 bits, two or four times a unit. out: added to, [block]
 // [tile][value]: SPLIT rows g, g + 8 of batch row 4 tile + q; else (row, batch row 8 tile + 2q + 0 / 1).
 template <int MT, int BLK, bool SPLIT, bool GRP>
 __device__ __forceinline__ void x_decode2(const uint8_t* codes, const uint8_t* bt, const uint8_t* vt, const uint8_t* sc,
                                           const float* fold, const float* sx, bool bias, const float (&al)[2 * BLK],
                                           int g, int q, int lane, const XParams& P,
-                                          float (&run)[BLK][MT][SPLIT ? 2 : 4]) {
-  constexpr int R = 2 * BLK, NV = SPLIT ? 2 : 4;
+                                          float (&out)[BLK][MT][SPLIT ? 2 : 4]) {
+  constexpr int R = 2 * BLK;
   // The steps alternate between two sets of accumulators: half the chain, and MMAs that do not wait for one
   // another (14b layer, M = 16: 54.3 -> 53.2 us); with one tile and v in A one set folded twice as often is
   // faster (M = 8: 39.1 us; 40.2 with two).
-  constexpr bool kTwo = SPLIT || GRP || MT > 1;
-  constexpr int kFold = GRP ? 2 : (SPLIT ? 8 : (kTwo ? 4 : 2));  // words (four steps each) per fold
-  float acc[2][BLK][MT][4], part[BLK][MT][NV];
-#pragma unroll
-  for (int k = 0; k < BLK; ++k)
-#pragma unroll
-    for (int j = 0; j < MT; ++j)
-#pragma unroll
-      for (int z = 0; z < NV; ++z) part[k][j][z] = 0.f;
-#pragma unroll (SPLIT || (MT == 1 && !GRP) ? 8 : (GRP ? 2 : 4))  // registers
+  constexpr bool kTwo = SPLIT ? MT == 1 : (GRP || MT > 1);  // (split tiles beyond the first: registers)
+  constexpr int kFold = GRP || !kTwo ? 2 : 4;                // words (four steps each) per fold
+  float acc[2][BLK][MT][4];
+#pragma unroll (MT == 1 && (SPLIT || !GRP) ? 8 : (GRP ? 2 : 4))  // registers
   for (int w = 0; w < 8; ++w) {
     uint32_t c[R];
 #pragma unroll
@@ -940,28 +934,20 @@ __device__ __forceinline__ void x_decode2(const uint8_t* codes, const uint8_t* b
       for (int j = 0; j < MT; ++j) {
         const float *d = &acc[0][r >> 1][j][2 * (r & 1)], *e = &acc[1][r >> 1][j][2 * (r & 1)];
         if constexpr (SPLIT) {
-          float& t = GRP ? part[r >> 1][j][r & 1] : run[r >> 1][j][r & 1];
-          const float sum = fmaf(d[1] + e[1], kXLo, d[0] + e[0]) * fold[4 * j + q];
+          float& t = out[r >> 1][j][r & 1];
+          const float sum = (kTwo ? fmaf(d[1] + e[1], kXLo, d[0] + e[0]) : fmaf(d[1], kXLo, d[0])) * fold[4 * j + q];
           if (GRP) t += fmaf(a1, sum, bias ? be * sx[16 * blk + 4 * j + q] : 0.f);
           else t = fmaf(a1, sum, t);
         } else {
 #pragma unroll
           for (int z = 0; z < 2; ++z) {
-            float& t = run[r >> 1][j][2 * (r & 1) + z];
+            float& t = out[r >> 1][j][2 * (r & 1) + z];
             if (GRP) t += fmaf(a1, d[z] + e[z], bias ? be * sx[16 * blk + 8 * j + 2 * q + z] : 0.f);
             else t = fmaf(a1, kTwo ? d[z] + e[z] : d[z], t);
           }
         }
       }
     }
-  }
-  if constexpr (GRP && SPLIT) {
-#pragma unroll
-    for (int k = 0; k < BLK; ++k)
-#pragma unroll
-      for (int j = 0; j < MT; ++j)
-#pragma unroll
-        for (int z = 0; z < NV; ++z) run[k][j][z] += part[k][j][z];
   }
 }
 
@@ -1112,6 +1098,10 @@ __global__ void __launch_bounds__(kXThreads, 1)
     qtea_gemv_mma_kernel(const __grid_constant__ TensorMaps maps, const __grid_constant__ XParams P) {
   constexpr bool BASE3 = MODE <= kXRows, DIAG = MODE == kXDiag, VENC = MODE == kXV2;
   constexpr int NV = VENC ? 4 : 2;  // values of a thread per row block and tile
+  // 2-bit codes with v*x split: a unit's sum, residual included, is formed on its own before it joins the tile's, one
+  // rounding beside the tile's sum for 512 columns (Qwen3-14B layer, M = 4: errors of 0.80e-7 against 0.90e-7 of the
+  // outputs' norm and 32.8 against 32.4 us, with the accumulators folded twice a unit; the kernel before: 0.82e-7)
+  constexpr bool kUnit = MODE == kXSplit2;
   // SETS sets of H helper warps take units in turn; CW consumer warps of BLK 16-row blocks
   constexpr int H = kXHelpers, SETS = kXSets, BLK = kXBlocks, CW = kXTileRows / 16 / BLK;
   constexpr int kXHelperThreads = 32 * H;
@@ -1325,9 +1315,19 @@ __global__ void __launch_bounds__(kXThreads, 1)
     const int off = BASE3 ? (int)(((size_t)(tr + g) * a.row_bytes + (size_t)c.ch * kXChunkBytes) & 15) : 0;
     const uint8_t* row = sb + (tr + g) * row_slot;
     const int rsn = x_res_steps(c, cur);
+    float unit[BLK][MT][NV];
+    if constexpr (kUnit) {
+#pragma unroll
+      for (int k = 0; k < BLK; ++k)
+#pragma unroll
+        for (int j = 0; j < MT; ++j)
+#pragma unroll
+          for (int z = 0; z < NV; ++z) unit[k][j][z] = 0.f;
+    }
+    float (&sums)[BLK][MT][NV] = kUnit ? unit : run;
     if constexpr (!BASE3) {
       x_decode2<MT, BLK, !VENC, GRP>(sb + (tr + g) * kChunkRowBytes + 4 * q, sb + lay.b, sb + lay.v, sc, fold, sx,
-                                     a.bias != 0, al, g, q, lane, P, run);
+                                     a.bias != 0, al, g, q, lane, P, sums);
     } else if constexpr (DIAG) {
       // the lane's block: 2^-E, alpha, and beta times its sum of x
       const int o0 = off + 26 * q;
@@ -1362,7 +1362,15 @@ __global__ void __launch_bounds__(kXThreads, 1)
 #pragma unroll
         for (int j = 0; j < MT; ++j)
 #pragma unroll
-          for (int z = 0; z < NV; ++z) run[k][j][z] += acc[k][j][VENC ? z : 2 * z];
+          for (int z = 0; z < NV; ++z) sums[k][j][z] += acc[k][j][VENC ? z : 2 * z];
+    }
+    if constexpr (kUnit) {
+#pragma unroll
+      for (int k = 0; k < BLK; ++k)
+#pragma unroll
+        for (int j = 0; j < MT; ++j)
+#pragma unroll
+          for (int z = 0; z < NV; ++z) run[k][j][z] += unit[k][j][z];
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(smem_u32(&empty[st]));

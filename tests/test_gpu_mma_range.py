@@ -169,3 +169,15 @@ def test_row_scales_far_apart(qt, fmt, M, massive):
     y_ref, bound = oracle.gemv(p.x, p.T, p.alpha, p.v, p.salient_idx, p.residual_vals, p.residual_idx, group_size=128)
     err = np.abs(call(qt, p, fmt, False, False) - y_ref)
     assert np.all(err <= REL * bound), f"worst {np.nanmax(err / np.maximum(bound, 1e-30)):.3g} of the bound"
+
+
+@pytest.mark.parametrize("M", [5, 9, 16])
+@pytest.mark.parametrize("K,group,bias", [(256, 128, True), (370, 128, True), (768, 128, False), (700, 0, True)])
+def test_small_errors_where_sums_were_fp32(qt, M, K, group, bias):
+    """2-bit calls at M >= 5 with a scale map of no whole 16-byte vectors, or one beta per row: products of 11 bits
+    (v*x split), not of 22, whose truncated sums leave 1.1e-7 of the outputs' norm; fp32 sums leave 0.75e-7 to 0.9e-7."""
+    p = synth.make_problem("small", 2048, K, M, 0, seed=K + M, group_size=group, beta_std=0.002 if bias else 0.0)
+    y_ref, _ = oracle.gemv(p.x, p.T, p.alpha, p.v, p.salient_idx, p.residual_vals, p.residual_idx,
+                           beta=p.beta if bias else None, group_size=group or K)
+    y = call(qt, p, "2bit", bias, False)
+    assert np.linalg.norm(y - y_ref) <= 0.8e-7 * np.linalg.norm(y_ref)
