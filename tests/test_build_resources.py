@@ -92,3 +92,15 @@ def test_narrow_row_resident_instantiations_fit_two_ctas_per_sm(kernels):
     assert len(narrow) == 4 and len(wide) == 2
     assert all(regs <= 128 for regs, _, _ in narrow.values())  # 2 x 256 threads x 128 = 65,536
     assert all(regs <= 255 for regs, _, _ in wide.values())
+
+
+def test_tensor_core_kernel_is_reported_and_spills_nothing(kernels):
+    """Every form of the kernel with staged B operands: base-3 at M = 1 and in one to four tiles, 2-bit split without scale
+    groups and in one to four tiles with them, and with v in A in one or two tiles; 512 threads of at most 128
+    registers fill an SM."""
+    mma = {n: v for n, v in kernels.items() if "qtea_gemv_mma_kernel" in n}
+    forms = sorted(re.search(r"kernelILi(\d)ELi(\d)ELb([01])E", n).groups() for n in mma)
+    assert forms == sorted([("1", "0", "1")] + [(t, "1", "1") for t in "1234"] + [("1", "2", "0")] +
+                           [(t, "2", "1") for t in "1234"] + [(t, "3", g) for t in "12" for g in "01"])
+    for name, (regs, st, ld) in mma.items():
+        assert st == 0 and ld == 0 and regs <= 128, name
