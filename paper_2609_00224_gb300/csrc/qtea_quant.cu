@@ -339,7 +339,9 @@ __device__ __forceinline__ float divide(float d, float a, float y) {
 // lie in [2^-40, 2^40], v alpha / 2 = v (alpha / 2) and a term that counts has |W - beta| above 2^-81, so
 // divide() holds below 2^60; the rest is done again with the general operations. The first CTA of a launch
 // with s > 0 selects the salient columns instead, beside the sums. 16 warps where there is a CTA per SM at
-// most (the chain of additions bounds: 4 cycles a row), 8 with three CTAs per SM above. Measured per round: 60
+// most (the chain of additions bounds, 4 cycles a row if it had its issue slots alone; measured 11.6 at 4096 x 4096:
+// three forming warps share the adding warp's scheduler), 8 and two CTAs per SM above (shared memory: a third lacks
+// 1.4 KB). Measured per round: 60
 // us at 4096 x 14336 (235 MB of W: 3.9 TB/s), 23 us at 4096 x 4096; with W and alpha, beta read through
 // registers a tile ahead, a library division per term and one column per lane 111 and 47 us. The whole
 // quantizer (groups of 128 with beta, four refits, two rounds, s = 3 % of K) 837 -> 249 us at 4096 x 14336.
@@ -350,6 +352,10 @@ struct QColSmem {
   float term[2][kTile / 4][32][4];
   float4 scale[kStages][kTile];
 };
+
+// Two of the smaller CTAs fit in an SM's 228 KB (1 KB of each is the system's; counts and the selection's sums are static);
+// their registers are kept to what three would have, 80: with more, 247.6 -> 251.2 us for the quantizer at 4096 x 14336.
+static_assert(2 * (sizeof(QColSmem<8>) + 1024 + 512) <= 228 * 1024, "two CTAs per SM");
 
 template <int WARPS>
 __global__ void __launch_bounds__(WARPS * 32, WARPS == 8 ? 3 : 1) quant_colsum_kernel(
