@@ -629,7 +629,7 @@ bool mb_capable(const qtea_layout* l, int M) {
   if (!l->mb_ok || !l->m1_ok || M < 1 || M > 16) return false;
   if (!is_paper(l)) return M >= 2;
   if (l->format != QTEA_FMT_2BIT) return false;
-  return l->group_size == 128 || !(l->options & QTEA_OPT_BIAS);
+  return l->group_size != l->K || !(l->options & QTEA_OPT_BIAS);  // one group per row (K = 128 too): alpha alone
 }
 
 // Low-batch dispatch: as many consecutive problems per launch as fit (one kernel variant per

@@ -100,3 +100,16 @@ def test_grouped_with_sparse_ones(qt, fmt, M):
         assert plan == [base3_kernel(M), "base3_mma", base3_kernel(M), base3_kernel(M)]
     for (p, _), y in zip(items, qt.qtea_gemv_grouped([q for _, q in items])):
         check(p, y)
+
+
+@pytest.mark.parametrize("fmt", ["base3", "2bit"])
+@pytest.mark.parametrize("M", [1, 2, 4, 5, 16])
+@pytest.mark.parametrize("s", [8, 64])
+@pytest.mark.parametrize("fp8", [False, True])
+@pytest.mark.parametrize("bias", [False, True])
+def test_one_group_of_128_columns(qt, fmt, M, s, fp8, bias):
+    """K = 128: groups of 128 columns are one group per row, and the scales pairs with beta."""
+    p, q = problem(qt, fmt, 260, 128, M, s, 128, bias, fp8, seed=3 * M + s)
+    y = qt.qtea_gemv(**q)
+    torch.cuda.synchronize()
+    check(p, y)
