@@ -15,8 +15,8 @@
 //    the same two bits.
 //  * B (activations): v*x is exact in fp32; times 2^E (E per chunk and batch row, so that the largest
 //    is below 2^15 after the halving that 2T asks for) it is held as two fp16 columns, hi and lo, whose
-//    sum hi + lo / 2^11 is exact down to 2^-28 of the chunk's largest. What it lacks of smaller products, infinities
-//    and NaN are added in fp32 at the end of the tile, to the rows whose code there is not 0. Four batch
+//    sum hi + lo / 2^11 is exact down to 2^-28 of the chunk's largest. Products 2^24 times the chunk's mean, infinities
+//    and NaN are left out and added in fp32 at the end of the tile, to the rows whose code there is not 0. Four batch
 //    rows make one n8 tile. The sums are folded with 2^-E per chunk. 2-bit codes at
 //    M >= 5 have v in A instead (2T * v, one exact fp16 multiply) and x in B, eight batch rows to a tile: half the
 //    MMAs (at M = 16 the decoding loop alone runs at 38 weights per clock per SM, with four split tiles at 27). From
@@ -47,9 +47,10 @@
 // the decoding (34.1 us where two give 32.6).
 // Measured, Llama3-8B layer in the paper's storage, seven GEMVs in one call: M = 1 82.4 -> 30.8 us (table
 // lookup before), M = 4 271 -> 34.8 us (fixed-point dp4a before), M = 16 6430 -> 71 us (the general kernel).
-// Qwen3-14B layer, 2-bit codes: M = 4 41.0 -> 32.5 us, M = 16 55.4 -> 53.2 us. (With the remainder in lo itself and no
-// search for products below its range, 30.4, 34.3, 71.3 and 32.3 us, and errors up to 2^-39 of a chunk's largest
-// product: 1 to 2 % of a row's sum |x W^| where activations of 5e-7 stand beside one of 6e4 whose code is 0.) Before, the kernel of
+// Qwen3-14B layer, 2-bit codes: M = 4 41.0 -> 32.8 us, M = 16 55.4 -> 53.4 us. (With the remainder in lo itself and no
+// product left out, 30.4, 34.3, 71.3 and 32.3 us, and errors up to 2^-39 of a chunk's largest product: 1 to 3 % of a
+// row's sum |x W^| where activations of 5e-7 stand beside one of 6e4 whose code is 0.) The same times with two activations
+// of 300, or 6e4 beside N(0, 0.1); with 6e4 beside N(0, 0.001), 46, 87, 296 and 95 us. Before, the kernel of
 // qtea_gemv_mb.cu, whose pass before the kernel and barrier across the grid this one does without: the barrier's
 // target was part of the launch, so that replays of a captured graph did not wait (34.5 and 49.5 us, and
 // other results than the direct call wherever the activations had changed).
@@ -198,8 +199,8 @@ __device__ __forceinline__ uint32_t x_b_offset(int c) {
 
 __device__ __forceinline__ bool x_finite(uint16_t h) { return (h & 0x7C00u) != 0x7C00u; }
 
-// Sixteen columns of x (rows m0, m0 + step, ...) and v per lane: columns 16 lane .. 16 lane + 15 of chunk ch; past K
-// x is zero and v one, and x zero from row M on.
+// Sixteen columns of x (rows m0, m0 + step, ...) and v per lane: columns 16 lane .. 16 lane + 15 of chunk ch, zero
+// past K and from row M on.
 template <int R>
 struct XRows {
   uint32_t x[R][8], v[8];
@@ -214,7 +215,7 @@ __device__ __forceinline__ void x_load_rows(const XProblem& a, int ch, int m0, i
     const int m = m0 + k * step;
     const uint16_t* src = k < 0 ? a.v + col : a.x + (size_t)m * a.K + col;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) d[i] = k < 0 && a.xv_vec ? 0x3C003C00u : 0u;
+    for (int i = 0; i < 8; ++i) d[i] = 0u;
     if (k < 0 ? !with_v : m >= M) continue;
     if (a.xv_vec) {  // rows of whole 16-byte vectors, 16-byte aligned
 #pragma unroll
@@ -226,15 +227,17 @@ __device__ __forceinline__ void x_load_rows(const XProblem& a, int ch, int m0, i
     } else {
 #pragma unroll
       for (int i = 0; i < 16; ++i)
-        d[i >> 1] |= (uint32_t)(col + i < a.K ? __ldg(src + i) : k < 0 ? (uint16_t)0x3C00 : (uint16_t)0) << (16 * (i & 1));
+        if (col + i < a.K) d[i >> 1] |= (uint32_t)__ldg(src + i) << (16 * (i & 1));
     }
   }
 }
 
 // v*x as an fp16 pair: f = v*x 2^(E - 1) below 2^15 (half of 2^E, since A is 2T), hi = f rounded, lo = the
 // remainder times 2^11, so that the pair is hi + lo / 2^11. f has 22 bits: above 2^-14 the pair is f itself (hi and
-// the remainder's 11 bits are normal, or the remainder is a multiple of 2^-35). What the pair lacks of smaller products
-// (2^-28 of the chunk's largest), and infinities and NaN, the consumers add in fp32 (x_left_out).
+// the remainder's 11 bits are normal, or the remainder is a multiple of 2^-35); below, that is 2^-28 of the largest, it is
+// off by 2^-36 at most, 2^(e - 50) for products below 2^(e + 1). E follows from the chunk's largest product, but no
+// further from the others than keeps that error below theirs in fp32: products of 2^(e + 1) and more, infinities and
+// NaN are left out of B and added by the consumers in fp32 (x_scan, x_left_out).
 constexpr float kXLo = 0x1p-11f;
 // The product of the two fp16 halves i (0: low), exact in fp32, and a half's addition to an fp32 sum: mixed-precision
 // instructions (PTX ISA 8.6, sm_100 and up), one each where two conversions and the operation would be two or three.
@@ -264,17 +267,10 @@ __device__ __forceinline__ void x_pair(float p0, float p1, float sc, __half2& hi
 // 2 |p| in the float's bits, without the sign: 0 for zero, from kXInf on infinities and NaN.
 __device__ __forceinline__ uint32_t x_mag(float p) { return __float_as_uint(p) << 1; }
 constexpr uint32_t kXInf = 0xFF000000u;
-// What the pair lacks of a product, sc = 2^(E - 1): exact, a multiple of fp16's smallest product 2^-48; infinities and
-// NaN whole.
-__device__ __forceinline__ float x_lacking(float p, float sc) {
-  if (x_mag(p) >= kXInf) return p;
-  __half2 hi, lo;
-  x_pair(p, 0.f, sc, hi, lo);
-  return fmaf(-__low2float(lo), kXLo, fmaf(p, sc, -__low2float(hi))) / sc;
-}
 // f(i, product i of the lane's sixteen) of batch row m in chunk ch, read from global memory eight columns at a time: for
 // what runs rarely, in functions of its own. (As part of the kernel's loops that code cost a call of one unit per CTA
-// 0.3 us and the Llama3-8B layer in the paper's storage up to 6, although it never ran.)
+// 0.3 us and the Llama3-8B layer in the paper's storage up to 6, although it never ran; at the tile's end, as calls, it
+// costs three calls of small layers at M = 11 0.3 us each.)
 template <typename F>
 __device__ __forceinline__ void x_products(const XProblem& a, int ch, int m, int lane, const F& f) {
 #pragma unroll 1
@@ -311,54 +307,53 @@ __device__ __forceinline__ int x_lane() {
 // A row's factors from e, the binade of its largest |v*x| (< 2^(e + 1)).
 __device__ __forceinline__ float x_sc(int e) { return __uint_as_float((uint32_t)(127 + 14 - e) << 23); }    // 2^(E - 1)
 __device__ __forceinline__ float x_fold(int e) { return __uint_as_float((uint32_t)(127 - 15 + e) << 23); }  // 2^-E
-__device__ __forceinline__ int x_binade(float lmax) {  // lmax: the lane's largest; 128 with an infinity or NaN
-  const uint32_t amax = __reduce_max_sync(0xffffffffu, __float_as_uint(lmax));
+__device__ __forceinline__ uint32_t x_largest(float lmax) {  // bits of the largest |v*x| over the lanes
+  return __reduce_max_sync(0xffffffffu, __float_as_uint(lmax));
+}
+__device__ __forceinline__ int x_binade(uint32_t amax) {  // 128 for an infinity or NaN, 0 for zero
   return amax ? (int)(amax >> 23) - 127 : 0;
 }
-// The least |v| of the lane's sixteen columns, in fp16 bits.
-__device__ __forceinline__ uint32_t x_least(const uint32_t (&v)[8]) {
-  uint32_t m = v[0] & 0x7FFF7FFFu;
-#pragma unroll
-  for (int i = 1; i < 8; ++i) m = __vminu2(m, v[i] & 0x7FFF7FFFu);
-  return min(m & 0xFFFFu, m >> 16);
-}
-// The lane's pairs may lack something (then x_search looks): not when the least |v| times fp16's smallest x, 2^-24,
-// or else the row's least x but for zeros, is at least 2^-28 of the binade 2^e. The first spares most chunks the
-// second: 2^e <= 16 with v near 1.
-__device__ __forceinline__ int x_exponent(uint32_t h) { return h >= 0x400u ? (int)(h >> 10) - 15 : -24; }
-__device__ __forceinline__ bool x_maybe(int e, uint32_t least_v, const uint32_t (&x)[8]) {
-  const int room = e - 28 - x_exponent(least_v);
-  if (room <= -24) return false;
-  uint32_t m = 0xFFFFFFFFu;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) m = __vminu2(m, __vsub2(x[i] & 0x7FFF7FFFu, 0x00010001u));  // zeros wrap to the top
-  return room > x_exponent(min(m & 0xFFFFu, m >> 16) + 1u);
+// The row may need another E (then x_search looks): with an infinity or NaN, or unless of the lanes with columns at
+// least half (rounded up) hold a product of 2^-20 of the largest, beside which an error of 2^-50 of it is nothing.
+__device__ __forceinline__ bool x_maybe(uint32_t amax, float lmax, int half) {
+  const uint32_t low = amax > 20u << 23 ? amax - (20u << 23) : 0u;
+  return amax >= 0x7F800000u || __popc(__ballot_sync(0xffffffffu, __float_as_uint(lmax) >= low)) < half;
 }
 
-// Binade of a row's finite products (returned with 2 e + lacking: some pair lacks something), by a warp.
-__device__ __forceinline__ int x_scan(const XProblem& a, int ch, int m, int lane, bool* not_finite) {
+// Products left out of a row of binade e: 2^(e + 1) and more, infinities and NaN.
+__device__ __forceinline__ bool x_outside(float p, int e) { return x_mag(p) >= (uint32_t)(128 + e) << 24; }
+// The binade of a row, by a warp: that of its largest finite product, but at most 24 above the mean binade of those that
+// are not zero. The pairs' error, 2^(e - 50), is then below 2^-26 of that mean; an fp32 sum rounds at 2^-24 of itself.
+__device__ __forceinline__ int x_scan(const XProblem& a, int ch, int m, int lane, bool* rebuild) {
   float lmax = 0.f;
-  uint32_t lmin = 0xFFFFFFFFu;
+  int sum = 0, n = 0;
   bool inf = false;
   x_products(a, ch, m, lane, [&](int, float p) {
-    lmin = min(lmin, x_mag(p) - 1u);  // zeros wrap to the top
-    if (x_mag(p) < kXInf) lmax = fmaxf(lmax, fabsf(p));
-    else inf = true;
+    const uint32_t mag = x_mag(p);
+    if (mag >= kXInf) {
+      inf = true;
+    } else if (mag) {
+      lmax = fmaxf(lmax, fabsf(p));
+      sum += (int)(mag >> 24) - 127;
+      ++n;
+    }
   });
-  const int e = x_binade(lmax);
-  *not_finite = __any_sync(0xffffffffu, inf);
-  return 2 * e + (__any_sync(0xffffffffu, inf || lmin < ((uint32_t)(127 - 28 + e) << 24) - 1u) ? 1 : 0);
+  const int top = x_binade(x_largest(lmax));
+  sum = __reduce_add_sync(0xffffffffu, sum);
+  n = __reduce_add_sync(0xffffffffu, n);
+  const int e = n ? min(top, (sum >= 0 ? sum / n : -((n - 1 - sum) / n)) + 24) : 0;
+  *rebuild = __any_sync(0xffffffffu, inf) || e < top;
+  return e;
 }
-// After batch row m of a chunk has been built: true when its pairs lack something. With infinities or NaN among the
-// products the row is built again, with the finite ones' factor and zeros in their places (layouts: x_build_row and
-// x_build_row2).
+// After batch row m of a chunk has been built from its largest product: true when it has been built again with zeros in
+// the places of products that are left out (layouts: x_build_row and x_build_row2).
 template <bool BASE3, bool DIAG>
 __device__ __noinline__ bool x_search(const XProblem& a, int ch, int m, float* fold, const uint32_t* boff, uint8_t* bt) {
   const int lane = x_lane();
-  bool not_finite;
-  const int es = x_scan(a, ch, m, lane, &not_finite);
-  if (!not_finite) return es & 1;
-  const float sc = x_sc(es >> 1);
+  bool rebuild;
+  const int e = x_scan(a, ch, m, lane, &rebuild);
+  if (!rebuild) return false;
+  const float sc = x_sc(e);
   const int q = lane >> 3, w = lane >> 2, n = BASE3 ? (DIAG ? 2 * q : 2 * (m & 3)) : (2 * (m & 3)) ^ (w & 3);
   uint8_t* base = bt + (BASE3 ? (DIAG ? 8 * q : (m >> 2) * kXBTileBytes + 2048 * q)
                               : (m >> 2) * kXTile2Bytes + w * 1024 + (lane & 3) * 8);
@@ -370,21 +365,21 @@ __device__ __noinline__ bool x_search(const XProblem& a, int ch, int m, float* f
       o = DIAG ? o & 0x3FFFu : (o & 0x1FFFu) + (o & 0x2000u ? 8192 - 2048 * q + 8 * q : 0);
     }
     __half2 hi, lo;
-    x_pair(x_mag(p) < kXInf ? p : 0.f, 0.f, sc, hi, lo);
+    x_pair(x_outside(p, e) ? 0.f : p, 0.f, sc, hi, lo);
     *reinterpret_cast<__half*>(base + o + 32 * col) = __low2half(hi);
     *reinterpret_cast<__half*>(base + o + 32 * (col ^ 1u)) = __low2half(lo);
   });
-  if (lane == 0) fold[m] = x_fold(es >> 1);
+  if (lane == 0) fold[m] = x_fold(e);
   return true;
 }
 
 // One batch row's B operand of a chunk, by one warp (lane = 16 columns; boff: the block's places, two
-// columns a word). True when the lane's pairs may lack something. DIAG (M =
+// columns a word). True when the row may need another E. DIAG (M =
 // 1): column pair q of the tile for block q, else column pair m % 4. The factor 2^-E and the blocks'
 // sums of x go to fold[m] and sx[block][m].
 template <bool DIAG>
 __device__ __forceinline__ bool x_build_row(const uint32_t (&x)[8], const uint32_t (&v)[8], int m, const uint32_t* boff, uint8_t* bt, float* fold,
-                                            float* sx, uint32_t least_v, int lane) {
+                                            float* sx, int half, int lane) {
   // v*x is exact in fp32; formed here for the largest and again below (sixteen registers fewer)
   auto product = [&](int i) { return x_fma16(x_half(v[i >> 1], i & 1), x_half(x[i >> 1], i & 1), 0.f); };
   float sum = 0.f, lmax = 0.f;
@@ -393,7 +388,8 @@ __device__ __forceinline__ bool x_build_row(const uint32_t (&x)[8], const uint32
     sum = x_add16(x_half(x[i >> 1], i & 1), sum);
     lmax = x_max_nan(lmax, fabsf(product(i)));
   }
-  const int e = x_binade(lmax);
+  const uint32_t amax = x_largest(lmax);
+  const int e = x_binade(amax);
   const float sc = x_sc(e);
   if (lane == 0) fold[m] = x_fold(e);
   const int q = lane >> 3, n = DIAG ? 2 * q : 2 * (m & 3);  // the lane's block, the hi column
@@ -417,7 +413,7 @@ __device__ __forceinline__ bool x_build_row(const uint32_t (&x)[8], const uint32
   sum += __shfl_xor_sync(0xffffffffu, sum, 2);
   sum += __shfl_xor_sync(0xffffffffu, sum, 4);
   if ((lane & 7) == 0) sx[16 * q + m] = sum;
-  return x_maybe(e, least_v, x);
+  return x_maybe(amax, lmax, half);
 }
 
 // 2-bit codes: one batch row's B operand of a chunk, by one warp. The lane's 16 columns are one code word, W =
@@ -427,7 +423,7 @@ __device__ __forceinline__ bool x_build_row(const uint32_t (&x)[8], const uint32
 // else column m % 8 of tile m / 8 holds x itself. SUM: the groups' sums of x too (for beta).
 template <bool SPLIT, bool SUM>
 __device__ __forceinline__ bool x_build_row2(const uint32_t (&x)[8], const uint32_t (&v)[8], int m, uint8_t* bt, float* fold,
-                                             float* sx, uint32_t least_v, int lane) {
+                                             float* sx, int half, int lane) {
   const int q = lane & 3, w = lane >> 2, key = w & 3;
   float sum = 0.f;
   uint8_t* base = bt + (SPLIT ? m >> 2 : m >> 3) * kXTile2Bytes + w * 1024 + q * 8;
@@ -440,10 +436,11 @@ __device__ __forceinline__ bool x_build_row2(const uint32_t (&x)[8], const uint3
       if (SUM) sum = x_add16(x_half(x[i >> 1], i & 1), sum);
       lmax = x_max_nan(lmax, fabsf(product(i)));
     }
-    const int e = x_binade(lmax);
+    const uint32_t amax = x_largest(lmax);
+    const int e = x_binade(amax);
     const float sc = x_sc(e);
     if (lane == 0) fold[m] = x_fold(e);
-    maybe = x_maybe(e, least_v, x);
+    maybe = x_maybe(amax, lmax, half);
     const int n = (2 * (m & 3)) ^ key;
 #pragma unroll
     for (int T = 0; T < 4; ++T) {
@@ -951,21 +948,22 @@ __device__ __forceinline__ void x_decode2(const uint8_t* codes, const uint8_t* b
   }
 }
 
-// What B lacks of batch row m in chunk ch: the sum of alpha T x_lacking(v*x) in fp32, and of the residual's values times
+// What B leaves out of batch row m in chunk ch: the sum of alpha T (v*x) in fp32, and of the residual's values times
 // x where x is not finite, for the thread's rows row0, row0 + 8, + 16, + 24. Everything is read from global memory
-// again: two passes over the chunk to find the columns, some 500 cycles for each. Rare (an activation 2^28
-// times another one of its chunk).
+// again: two passes over the chunk to find the columns, some 500 cycles for each. Rare (an activation 2^24
+// times the chunk's mean).
 template <bool BASE3, bool DIAG>
 __device__ __noinline__ float4 x_left_out(const XProblem& a, int ch, int m, int row0) {
   constexpr int R = 2 * kXBlocks;
   const int lane = x_lane();
   const uint16_t* xm = a.x + (size_t)m * a.K;
-  bool not_finite;
-  const float sc = x_sc(x_scan(a, ch, m, lane, &not_finite) >> 1);
+  bool rebuild;
+  const int e = x_scan(a, ch, m, lane, &rebuild);
   uint32_t mask = 0u;
-  x_products(a, ch, m, lane, [&](int i, float p) {
-    if (x_lacking(p, sc) != 0.f) mask |= 1u << i;  // a NaN too
-  });
+  if (rebuild)
+    x_products(a, ch, m, lane, [&](int i, float p) {
+      if (x_outside(p, e)) mask |= 1u << i;
+    });
   float out[R];
 #pragma unroll
   for (int r = 0; r < R; ++r) out[r] = 0.f;
@@ -973,7 +971,7 @@ __device__ __noinline__ float4 x_left_out(const XProblem& a, int ch, int m, int 
     const int src = __ffs((int)lanes) - 1;
     const int k = ch * kXChunkCols + 16 * src + __ffs((int)__shfl_sync(0xffffffffu, mask, src)) - 1;
     if (lane == src) mask &= mask - 1u;
-    const float p = x_lacking(h2f(__ldg(a.v + k)) * h2f(__ldg(xm + k)), sc);
+    const float p = x_fma16(__ldg(a.v + k), __ldg(xm + k), 0.f);
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const int row = min(row0 + 8 * r, a.N - 1);  // rows past N: never written
@@ -1010,7 +1008,7 @@ __device__ __noinline__ float4 x_left_out(const XProblem& a, int ch, int m, int 
           int b = __ldg(codes + 24) + 243 * __ldg(codes + 25);
           for (int k = 128 * blk + 120; k < min(a.K, 128 * blk + 128); ++k, b /= 3) {
             const float p = x_fma16(__ldg(a.v + k), __ldg(xm + k), 0.f);
-            if (x_mag(p) < kXInf) sum = fmaf((float)(b % 3 - 1), p - x_lacking(p, sc), sum);  // what B holds of it
+            if (!x_outside(p, e)) sum = fmaf((float)(b % 3 - 1), p, sum);  // those that B holds
           }
         }
         sum *= h2f(al[r]);
@@ -1019,8 +1017,8 @@ __device__ __noinline__ float4 x_left_out(const XProblem& a, int ch, int m, int 
       }
     }
   }
-  const int e = ch * (a.res_q * a.n_chunks + a.res_r), st0 = e / a.n_chunks;
-  const int n_steps = a.res_q + (e - st0 * a.n_chunks + a.res_r >= a.n_chunks ? 1 : 0);
+  const int at = ch * (a.res_q * a.n_chunks + a.res_r), st0 = at / a.n_chunks;
+  const int n_steps = a.res_q + (at - st0 * a.n_chunks + a.res_r >= a.n_chunks ? 1 : 0);
   uint16_t xs = 0;
   if (x_has_sal(a, st0, n_steps, lane)) xs = x_at_sal(a, m, __ldg(a.sal + 16 * st0 + lane));
   for (uint32_t lanes = __ballot_sync(0xffffffffu, !x_finite(xs)); lanes; lanes &= lanes - 1u) {
@@ -1223,8 +1221,8 @@ __global__ void __launch_bounds__(kXThreads, 1)
           *reinterpret_cast<uint32_t*>(sb + lay.rpos + 4 * ht) = pos.b[0] | pos.b[1] << 8 | pos.b[2] << 16 | pos.b[3] << 24;
       }
       x_cp_arrive(smem_u32(&full[st]));
-      const uint32_t least_v = VENC ? 0u : x_least(rows.v);
-      uint32_t maybe = 0u;  // bit m: the pairs of batch row m may lack something; bit 16 + m: some x at a salient column does
+      const int half = (min(32, (a.K - c.ch * kXChunkCols + 15) / 16) + 1) / 2;
+      uint32_t maybe = 0u;  // bit m: batch row m may need another E; bit 16 + m: some x at a salient column is not finite
 #pragma unroll
       for (int k = 0; k < R; ++k) {
         const int m = hw + k * H;
@@ -1241,10 +1239,10 @@ __global__ void __launch_bounds__(kXThreads, 1)
                                        ((lane >> 4) * 32 + 4 * n + ((lane >> 2) & 3)) * 8 + 2 * (lane & 3)) = xs[k];
         float* fold = reinterpret_cast<float*>(sb + lay.fold);
         float* sx = reinterpret_cast<float*>(sb + lay.sx);
-        bool lacks;
-        if constexpr (BASE3) lacks = x_build_row<DIAG>(rows.x[k], rows.v, m, boff, sb + lay.b, fold, sx, least_v, lane);
-        else lacks = x_build_row2<!VENC, GRP>(rows.x[k], rows.v, m, sb + lay.b, fold, sx, least_v, lane);
-        if (lacks) maybe |= 1u << m;
+        bool look;
+        if constexpr (BASE3) look = x_build_row<DIAG>(rows.x[k], rows.v, m, boff, sb + lay.b, fold, sx, half, lane);
+        else look = x_build_row2<!VENC, GRP>(rows.x[k], rows.v, m, sb + lay.b, fold, sx, half, lane);
+        if (look) maybe |= 1u << m;
         if (VENC && m == 0) x_build_v(rows.v, sb + lay.v, lane);
       }
       if constexpr (!VENC) {

@@ -1,13 +1,13 @@
 """Activations of a wide range on the tensor-core kernel with staged B operands, against the fp64 oracle: one massive
 value per 512-column chunk beside activations down to 2^-36 of it, with codes 0 at the massive columns in part of
 the rows, where an error relative to the massive value shows. v*x is held as an fp16 pair, exact down to 2^-28 of
-the chunk's largest; what smaller products lack of it is added in fp32, as infinities and NaN are. (2-bit codes at M
->= 5 take 2T v in A instead, exact below |v| = 2^15; larger v are added in fp32 too.)
+the chunk's largest and within 2^-50 of it below; products 2^24 times the chunk's mean are taken out and added in fp32,
+as infinities and NaN are. (2-bit codes at M >= 5 take 2T v in A instead, exact below |v| = 2^15; with larger v the sum
+is formed in fp32.)
 
-Pass rule per element: |y - y_ref| <= 2e-6 * sum_j |x_j * W^[o][j]|, nothing absolute. Every product is exact; the
-tensor core truncates each of a chunk's at most 35 steps below 2^-24 of the partial sum, and what the pairs lack (up
-to 512 terms a chunk) joins in fp32, with partial sums that, over terms of either sign, stay a small part of the
-bound: 2e-6 is 34 roundings of the whole bound.
+Pass rule per element: |y - y_ref| <= 2e-6 * sum_j |x_j * W^[o][j]|, nothing absolute. The pairs' errors stay below 2^-26
+of a chunk's mean product; the tensor core truncates each of a chunk's at most 35 steps below 2^-24 of the partial
+sum, which over terms of either sign stays a small part of the bound: 2e-6 is 34 roundings of the whole bound.
 """
 import numpy as np
 import pytest
