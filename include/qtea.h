@@ -150,7 +150,8 @@ int qtea_pack_layout(const int8_t* ternary_codes, int N, int K, int group_size, 
  * tensor-core kernel 2T is exact and v*x an fp16 pair, exact down to 2^-28 of the largest of its 512 columns and within
  * 2^-50 of it below; columns 2^24 times the (geometric) mean and more are taken out and added in fp32. Products are
  * summed on the tensor cores over at most 512 columns, the rest in fp32 (a column where v*x is infinite or NaN counts
- * in the rows whose code there is not 0, or that hold its residual value); 2-bit layouts at M >= 5 take 2T*v and x in fp16 there, both exact, and where
+ * in the rows whose code there is not 0, or that hold its residual value); 2-bit layouts at M >= 5 with one alpha per row, or scale
+ * groups in rows of whole aligned 16-byte vectors, take 2T*v and x in fp16 there, both exact, and where
  * that gives no finite sum (|v| >= 32768, infinities and NaN) the sum is formed in fp32. The older low-batch
  * kernel takes 2T*v and x in fp16 too, which needs |v| < 32768; an infinity or NaN in x makes the batch row NaN. On the fixed-point
  * kernel (when v*x of the call fits in shared memory): the ternary sum is accumulated exactly in integers over 128-column blocks, with v*x in fixed point relative to the
